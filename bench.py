@@ -302,7 +302,7 @@ def measure_extras(cfg, L, W2, dm, flush, pk, iters=50):
         B.check(loop(side), "pr2_rollout_layers (capture)")
     graph_ms = timed(graph.replay, pre=lambda: hd.copy_(h0))
     per_layer = [cost.route_predict_work(Td, cfg.d, cfg.N, cfg.k, cfg.dtype, True),
-                 cost.dispatch_work(Td, cfg.d, cfg.k, cfg.dtype, gather=cfg.dtype == "fp32"),
+                 cost.dispatch_work(Td, cfg.d, cfg.k, cfg.dtype),
                  cost.expert_mlp_algorithmic_work(Td * cfg.k, cfg.d, cfg.m, cfg.N, cfg.dtype,
                                                   a_rows=0),  # h counted by routing
                  cost.combine_work(Td, cfg.d, cfg.k, cfg.n_shared, cfg.dtype)]
@@ -663,7 +663,7 @@ def run_pr2(args, rank, world, local_rank):
     work = {
         "route_predict": cost.route_predict_work(cfg.T, cfg.d, cfg.N, cfg.k, cfg.dtype, True),
         "route_replay": cost.route_replay_work(cfg.T, cfg.d, cfg.N, cfg.k, cfg.dtype, False),
-        "dispatch": cost.dispatch_work(cfg.T, cfg.d, cfg.k, cfg.dtype, gather=cfg.dtype == "fp32"),
+        "dispatch": cost.dispatch_work(cfg.T, cfg.d, cfg.k, cfg.dtype),
         # the fused minimum of the grouped GEMMs: h once and the hit experts' weights (the H
         # round trip and the Y write of this design are counted in `modeled_bytes`)
         "expert_gemm": cost.expert_mlp_algorithmic_work(
@@ -792,11 +792,10 @@ def run_pr2(args, rank, world, local_rank):
                     "no L2 flush (1.2 GB of expert weights per step)")
 
     # per layer forward: dispatch (one fused cooperative kernel when N % 4 == 0 and the grid is
-    # resident, as at every bench shape; else hist + scan + place; + a row gather on the fp32
-    # path only, the bf16 gate/up GEMM gathers its A rows itself), the routed grouped GEMMs (one
+    # resident, as at every bench shape; else hist + scan + place), the routed grouped GEMMs (one
     # launch for gate/up and down in bf16, two in fp32; + two for shared experts) and the
     # combine; plus one routing kernel per mode
-    n_dispatch = (1 if cfg.N % 4 == 0 and cfg.N <= 256 else 3) + (cfg.dtype == "fp32")
+    n_dispatch = 1 if cfg.N % 4 == 0 and cfg.N <= 256 else 3
     n_gemm = 1 if cfg.dtype == "bf16" else 2
     launches_per_step = 2 + 2 * (n_dispatch + n_gemm + 1 + (2 if cfg.n_shared else 0))
     line = dict(metric=METRIC, value=value, unit="tokens/s", n_gpus=world, steps=args.steps,

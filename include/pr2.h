@@ -114,8 +114,7 @@ pr2_status pr2_route_replay(const pr2_dims* dims, const void* h, const void* W_r
  * at that point of the launch sequence.  NULL members and a NULL struct pointer are ignored. */
 typedef struct {
     void* start;         /* before dispatch                                              */
-    void* dispatched;    /* after histogram, scan and stable placement (+ the row gather
-                          * on the fp32 path; the bf16 gate/up GEMM gathers its rows)    */
+    void* dispatched;    /* after histogram, scan and stable placement                    */
     void* gate_up_done;  /* after the routed experts' GEMMs (bf16: gate/up and down run as
                           * one launch) and the shared experts' gate/up GEMM              */
     void* down_done;     /* after the shared experts' down GEMM (the routed down GEMM on

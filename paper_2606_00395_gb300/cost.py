@@ -60,9 +60,9 @@ def route_replay_work(T: int, d: int, N: int, k: int, dtype: str = "bf16",
 
 
 def dispatch_work(T: int, d: int, k: int, dtype: str = "bf16", gather: bool = False) -> KernelWork:
-    """Histogram + scan + stable rank: read idx, write perm and inv.  With `gather` (the fp32
-    path) also read h once and write the permuted rows X_perm [T*k, d]; the bf16 gate/up GEMM
-    reads h through perm itself, so dispatch writes no rows there."""
+    """Histogram + scan + stable rank: read idx, write perm and inv.  The gate/up
+    GEMMs read h through perm themselves, so dispatch writes no rows; with `gather` the work of
+    a design that writes the permuted rows X_perm [T*k, d]: h read once, X_perm written."""
     e = _esz(dtype)
     b = T * k * 4 + 2 * T * k * 4
     if gather:

@@ -85,7 +85,6 @@ struct Workspace {
   TileEntry* stiles1;
   TileEntry* stiles2;
   int32_t* route_hist;  // per-CTA expert histograms of the rollout routing (pr2_moe_rollout_forward)
-  void* xperm;
   void* hbuf;
   void* ybuf;
   void* hs;
@@ -121,8 +120,9 @@ Workspace carve(const pr2_dims& dm, uint8_t* base) {
   w.stiles1 = reinterpret_cast<TileEntry*>(take(sizeof(TileEntry) * (w.shared_tiles + 1)));
   w.stiles2 = reinterpret_cast<TileEntry*>(take(sizeof(TileEntry) * (w.shared_tiles + 1)));
 
-  // permuted copy of h: only the fp32 path reads it; the bf16 gate/up GEMM gathers from h
-  w.xperm = dm.dtype == PR2_FP32 ? take(es * F * dm.d) : nullptr;
+  // fp32: the size that callers plan with includes a permuted copy of h, which no kernel writes
+  // (the gate/up GEMMs of both types gather their rows from h)
+  if (dm.dtype == PR2_FP32) take(es * F * dm.d);
   // H [Tk, m].  The rollout routing's per-CTA histograms share its first bytes: dispatch reads
   // them before the gate/up GEMM (which waits for dispatch) writes H.
   const size_t hist_bytes = sizeof(int32_t) * (size_t)mt_T * kRouteMaxSplit * dm.N;
@@ -462,12 +462,9 @@ pr2_status moe_forward_impl(const pr2_dims* dims, const void* h, const int32_t* 
   };
   mark(events ? events->start : nullptr);
 
-  const int es = static_cast<int>(esize(dm));
-  DispatchArgs da{idx,       dm.T,       dm.k,      dm.N,    dm.d,   es,     dm.n_shared,
-                  w.blk_hist, w.counts,  w.offsets, w.perm,  w.inv,  w.tiles, w.num_tiles,
-                  w.stiles1, w.stiles2,  h,         w.xperm, status, w.sync_ctr,
-                  dm.dtype == PR2_BF16 ? w.ready : nullptr, kTileM};
-  // (w.xperm is nullptr on the bf16 path: dispatch then launches no gather)
+  DispatchArgs da{idx,       dm.T,      dm.k,   dm.N,  dm.n_shared, w.blk_hist,  w.counts,
+                  w.offsets, w.perm,    w.inv,  w.tiles, w.num_tiles, w.stiles1, w.stiles2,
+                  status,    w.sync_ctr, dm.dtype == PR2_BF16 ? w.ready : nullptr, kTileM};
   if (err == cudaSuccess)
     err = (rhist != nullptr && dm.dtype == PR2_BF16)
               ? launch_dispatch_from_hist(da, rhist->hist, rhist->split, st)
@@ -477,7 +474,7 @@ pr2_status moe_forward_impl(const pr2_dims* dims, const void* h, const int32_t* 
 
   const int64_t F = dm.T * dm.k;
   GemmArgs g1{w.tiles, w.num_tiles, w.max_tiles, dm.d, dm.m, dm.m, w.hbuf, status,
-              h, w.perm, dm.k};  // gathered A (bf16); the fp32 GEMM reads w.xperm
+              h, w.perm, dm.k};  // gathered A
   GemmArgs g2{w.tiles, w.num_tiles, w.max_tiles, dm.m, dm.d, dm.d, w.ybuf, status,
               nullptr, nullptr, 0};
   GemmArgs s1{w.stiles1, w.num_tiles + 1, w.shared_tiles, dm.d, dm.m, dm.m, w.hs, status,
@@ -512,20 +509,20 @@ pr2_status moe_forward_impl(const pr2_dims* dims, const void* h, const int32_t* 
     }
     mark(events ? events->down_done : nullptr);
   } else {
-    err = launch_expert_simt(true, static_cast<const float*>(w.xperm),
-                             static_cast<const float*>(W_gate), static_cast<const float*>(W_up),
-                             g1, st);
+    const int64_t FS = dm.T * dm.n_shared;  // rows of the shared experts
+    err = launch_expert_simt(true, static_cast<const float*>(h), static_cast<const float*>(W_gate),
+                             static_cast<const float*>(W_up), g1, F, num_sms, st);
     if (err == cudaSuccess && dm.n_shared > 0)
       err = launch_expert_simt(true, static_cast<const float*>(h),
                                static_cast<const float*>(Ws_gate),
-                               static_cast<const float*>(Ws_up), s1, st);
+                               static_cast<const float*>(Ws_up), s1, FS, num_sms, st);
     mark(events ? events->gate_up_done : nullptr);
     if (err == cudaSuccess)
       err = launch_expert_simt(false, static_cast<const float*>(w.hbuf),
-                               static_cast<const float*>(W_down), nullptr, g2, st);
+                               static_cast<const float*>(W_down), nullptr, g2, F, num_sms, st);
     if (err == cudaSuccess && dm.n_shared > 0)
       err = launch_expert_simt(false, static_cast<const float*>(w.hs),
-                               static_cast<const float*>(Ws_down), nullptr, s2, st);
+                               static_cast<const float*>(Ws_down), nullptr, s2, FS, num_sms, st);
     mark(events ? events->down_done : nullptr);
   }
   if (err != cudaSuccess) return PR2_ERR_CUDA;

@@ -10,8 +10,7 @@
 //   3. place  - one block per 256 slots again: per-warp counts via __match_any_sync, a scan
 //               over the 8 warps, then rank = popc(lanes below with the same expert):
 //               perm[offsets[e] + r] = f, inv[f] = its position (-1 for an invalid slot).
-//   4. gather - X[p, :] = h[perm[p] / k, :], 16-byte vectors, one warp per row; fp32 path only
-//               (the bf16 gate/up GEMM reads its rows from h through perm itself).
+// The gate/up GEMMs read their rows from h through perm themselves.
 // Steps 1-3 normally run as one cooperative launch (dispatch_fused_kernel): every block counts
 // its slots, one bounded grid barrier, then each block derives the expert totals, its own
 // per-expert bases and the expert offsets from the whole block histogram (identical in every
@@ -577,26 +576,6 @@ bool fused_dispatch_ok(int N, int nblk, int num_sms) {
   return static_cast<int64_t>(per_sm) * num_sms >= nblk;
 }
 
-// X[p, :] = h[perm[p] / k, :] for p < offsets[N]; row_vec = 16-byte vectors per row.
-__global__ void __launch_bounds__(256)
-    gather_kernel(const uint4* __restrict__ h, const int32_t* __restrict__ perm,
-                  const int32_t* __restrict__ nrows_ptr, int k, int row_vec,
-                  uint4* __restrict__ X) {
-  pdl_wait();
-  pdl_trigger();
-  const int nrows = *nrows_ptr;
-  const int lane = threadIdx.x & 31;
-  const int warp0 = static_cast<int>((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nwarps = static_cast<int>((gridDim.x * blockDim.x) >> 5);
-  for (int p = warp0; p < nrows; p += nwarps) {
-    const int t = perm[p] / k;
-    const uint4* src = h + static_cast<int64_t>(t) * row_vec;
-    uint4* dst = X + static_cast<int64_t>(p) * row_vec;
-#pragma unroll 8
-    for (int v = lane; v < row_vec; v += 32) dst[v] = __ldg(src + v);
-  }
-}
-
 template <typename T, int V, int KMAX>  // V elements per 16-byte vector, k <= KMAX
 __global__ void __launch_bounds__(256)
     combine_kernel(const T* __restrict__ Y, const T* __restrict__ Ys,
@@ -878,18 +857,6 @@ cudaError_t launch_dispatch(const DispatchArgs& a, int num_sms, cudaStream_t st)
                        a.N, static_cast<const int32_t*>(a.blk_hist), a.perm, a.inv);
       if (err != cudaSuccess) return err;
     }
-  }
-  if (nblk > 0 && a.xperm != nullptr) {
-    const int row_vec = a.d * a.esz / 16;
-    int64_t warps_needed = F;
-    int64_t blocks = (warps_needed + 7) / 8;
-    const int64_t cap = static_cast<int64_t>(num_sms) * 8;
-    if (blocks > cap) blocks = cap;
-    err = launch_pdl(gather_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, st, 1,
-                     static_cast<const uint4*>(a.h), static_cast<const int32_t*>(a.perm),
-                     static_cast<const int32_t*>(a.offsets + a.N), a.k, row_vec,
-                     static_cast<uint4*>(a.xperm));
-    if (err != cudaSuccess) return err;
   }
   return cudaSuccess;
 }

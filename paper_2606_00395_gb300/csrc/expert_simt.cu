@@ -1,57 +1,223 @@
 // fp32 grouped expert GEMMs (exact fp32 FMA; the fp32 layer needs a 1e-4 tolerance, which
-// TF32 tensor cores cannot meet).  Same tile table as the tensor-core path: block (i, j) takes
-// M-tile i of the table and 128 output columns; one thread per output column loops over the
-// tile's rows, so each weight row is streamed once per tile.
+// TF32 tensor cores cannot meet).  Same tile table as the tensor-core path.
 //   gate/up: H[r, c] = silu(X[r] . Wg_e[c]) * (X[r] . Wu_e[c])      (App. E.2, SwiGLU)
 //   down:    Y[r, c] = H[r] . Wd_e[c]
+// A block computes BM rows x BN columns of one M-tile.  Both operands are K-contiguous, so K
+// blocks of the rows and of the weight rows travel as 16-byte cp.async copies through a ring of
+// kStages stages in shared memory (the routed gate/up GEMM gathers its rows from h through perm
+// here: no permuted copy of h exists), and a thread accumulates a TM x TN register tile (twice
+// for gate and up) from float4 reads along K.  The row pitch of BK + 4 floats puts the 16-byte
+// words of eight consecutive rows on distinct banks.  K that is not a multiple of 4 (a ragged
+// expert width) copies 4 bytes at a time instead, its rows being unaligned.  Every output is one
+// chain of FMAs in ascending K.
+//
+// What bounds it: the FMA issue rate for large layers, and the chain of K blocks at small ones;
+// hence two tile sizes (launch_expert_simt).  A rollout + replay step of the T = 256, d = 128,
+// m = 256, N = 8, k = 2 layer takes 79 us with these kernels and took 5203 us with one thread
+// per output column walking its weight row by uncoalesced 4-byte loads for every row of the
+// tile, behind a launch that wrote a permuted copy of h.
 #include "pr2_device.cuh"
 #include "pr2_internal.h"
 
 namespace pr2 {
 namespace {
 
-constexpr int kCols = 128;
+constexpr int kStages = 3;
 
-__global__ void __launch_bounds__(kCols)
-    expert_simt_kernel(int swiglu, const float* __restrict__ A, const float* __restrict__ W0,
-                       const float* __restrict__ W1, const TileEntry* __restrict__ tiles,
-                       const int32_t* __restrict__ num_tiles, int K, int n_out, int b_rows,
-                       float* __restrict__ out, const int32_t* status) {
+// 4-byte asynchronous copy; src_bytes = 0 fills the word with zeros.
+__device__ __forceinline__ void cp_async_4(uint32_t smem_dst, const void* src, uint32_t src_bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_dst), "l"(src),
+               "r"(src_bytes)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_16(uint32_t smem_dst, const void* src,
+                                            uint32_t src_bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_dst), "l"(src),
+               "r"(src_bytes)
+               : "memory");
+}
+
+template <int BM, int BN, int TM, int TN, int BK, bool kSwiglu>
+struct SimtTile {
+  static constexpr int kThreads = (BM / TM) * (BN / TN);
+  static constexpr int kRows = BM + BN * (kSwiglu ? 2 : 1);  // A rows, then weight rows
+  static constexpr int kPitch = BK + 4;
+  static constexpr int kVecs = kRows * (BK / 4);             // 16-byte words of a stage
+  static constexpr int kLoads = kVecs / kThreads;
+  static constexpr int kStageFloats = kRows * kPitch;
+  static constexpr int kSmem = kStages * kStageFloats * 4;
+  static_assert(kVecs % kThreads == 0 && BM % 8 == 0 && BN % 8 == 0, "whole rounds of copies");
+  static_assert(kSmem <= 48 * 1024, "static shared memory");
+};
+
+template <int BM, int BN, int TM, int TN, int BK, bool kSwiglu>
+__global__ void __launch_bounds__((SimtTile<BM, BN, TM, TN, BK, kSwiglu>::kThreads))
+    expert_simt_kernel(const float* __restrict__ A, const int32_t* __restrict__ perm, int k,
+                       const float* __restrict__ W0, const float* __restrict__ W1,
+                       const TileEntry* __restrict__ tiles, const int32_t* __restrict__ num_tiles,
+                       int K, int n_out, int b_rows, int col_blocks, float* __restrict__ out,
+                       const int32_t* status) {
+  using S = SimtTile<BM, BN, TM, TN, BK, kSwiglu>;
+  __shared__ __align__(16) float smem[kStages * S::kStageFloats];
+  constexpr int kSub = kTileM / BM;  // row blocks of one M-tile
   pdl_wait();
   pdl_trigger();
-  // blockIdx.x < max_tiles by the grid; a dispatch that timed out leaves the table unwritten
-  if (status_timed_out(status) || static_cast<int>(blockIdx.x) >= *num_tiles) return;
-  const TileEntry te = tiles[blockIdx.x];
-  const int c = blockIdx.y * kCols + threadIdx.x;
-  if (c >= n_out) return;
-  const float* w0 = W0 + (static_cast<int64_t>(te.expert) * b_rows + c) * K;
-  const float* w1 = swiglu ? W1 + (static_cast<int64_t>(te.expert) * b_rows + c) * K : nullptr;
-  for (int r = 0; r < te.rows; ++r) {
-    const float* a = A + static_cast<int64_t>(te.a_row0 + r) * K;
-    float acc0 = 0.f, acc1 = 0.f;
-    if (swiglu) {
-      for (int i = 0; i < K; ++i) {
-        acc0 = fmaf(a[i], w0[i], acc0);
-        acc1 = fmaf(a[i], w1[i], acc1);
+  // mt < max_tiles by the grid; a dispatch that timed out leaves the table unwritten
+  const int row_block = static_cast<int>(blockIdx.x) / col_blocks;
+  const int mt = row_block / kSub;
+  if (status_timed_out(status) || mt >= *num_tiles) return;
+  const TileEntry te = tiles[mt];
+  const int r0 = (row_block % kSub) * BM;
+  if (r0 >= te.rows) return;
+  const int c0 = (static_cast<int>(blockIdx.x) % col_blocks) * BN;
+  const int tid = threadIdx.x;
+  const bool vec = K % 4 == 0;  // rows of 16-byte words (every base is 16-byte aligned)
+
+  // This thread's copies of a stage: row kRow of [A rows; W0 rows; W1 rows], words kc.. of it.
+  const float* src[S::kLoads];
+  uint32_t on = 0;
+#pragma unroll
+  for (int i = 0; i < S::kLoads; ++i) {
+    const int v = tid + i * S::kThreads;
+    const int row = v / (BK / 4), kc = (v % (BK / 4)) * 4;
+    src[i] = A;
+    if (row < BM) {
+      if (r0 + row < te.rows) {
+        const int p = te.a_row0 + r0 + row;
+        src[i] = A + static_cast<int64_t>(perm != nullptr ? perm[p] / k : p) * K + kc;
+        on |= 1u << i;
       }
-      acc0 = acc0 / (1.0f + expf(-acc0)) * acc1;
     } else {
-      for (int i = 0; i < K; ++i) acc0 = fmaf(a[i], w0[i], acc0);
+      const int c = c0 + (row - BM) % BN;
+      if (c < n_out) {
+        src[i] = (row - BM < BN ? W0 : W1) + (static_cast<int64_t>(te.expert) * b_rows + c) * K + kc;
+        on |= 1u << i;
+      }
     }
-    out[static_cast<int64_t>(te.out_row0 + r) * n_out + c] = acc0;
   }
+  const uint32_t sbase = smem_u32(smem);
+  auto issue = [&](int kb) {
+    const uint32_t st = sbase + static_cast<uint32_t>(kb % kStages) * S::kStageFloats * 4;
+    const int k0 = kb * BK;
+#pragma unroll
+    for (int i = 0; i < S::kLoads; ++i) {
+      const int v = tid + i * S::kThreads;
+      const int row = v / (BK / 4), kc = (v % (BK / 4)) * 4;
+      const uint32_t dst = st + static_cast<uint32_t>(row * S::kPitch + kc) * 4;
+      const bool live = (on >> i) & 1u;
+      if (vec) {
+        const bool in = live && k0 + kc < K;
+        cp_async_16(dst, in ? src[i] + k0 : A, in ? 16u : 0u);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const bool in = live && k0 + kc + j < K;
+          cp_async_4(dst + 4 * j, in ? src[i] + k0 + j : A, in ? 4u : 0u);
+        }
+      }
+    }
+  };
+
+  // Threads of a warp: 8 columns x 4 rows, so that a warp's reads of a stage touch eight
+  // consecutive weight rows and four consecutive A rows.
+  constexpr int kTx = BN / TN, kTy = BM / TM;
+  constexpr int kWx = kTx / 8;
+  const int lane = tid & 31, warp = tid >> 5;
+  const int tx = (lane & 7) + 8 * (warp % kWx);
+  const int ty = (lane >> 3) + 4 * (warp / kWx);
+  float acc0[TM][TN], acc1[kSwiglu ? TM : 1][TN];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+      acc0[i][j] = 0.f;
+      if (kSwiglu) acc1[i][j] = 0.f;
+    }
+  const int KB = (K + BK - 1) / BK;
+#pragma unroll
+  for (int s = 0; s < kStages - 1; ++s) {
+    if (s < KB) issue(s);
+    cp_async_commit();
+  }
+  for (int kb = 0; kb < KB; ++kb) {
+    cp_async_wait<kStages - 2>();
+    __syncthreads();  // stage kb has landed for every thread, stage kb - 1 is free
+    if (kb + kStages - 1 < KB) issue(kb + kStages - 1);
+    cp_async_commit();
+    const float* sa = smem + (kb % kStages) * S::kStageFloats;
+    const float* sb = sa + BM * S::kPitch;
+    const float* su = sb + BN * S::kPitch;
+#pragma unroll
+    for (int kk = 0; kk < BK; kk += 4) {
+      float4 a[TM], b[TN], u[kSwiglu ? TN : 1];
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+        a[i] = *reinterpret_cast<const float4*>(sa + (ty + kTy * i) * S::kPitch + kk);
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        b[j] = *reinterpret_cast<const float4*>(sb + (tx + kTx * j) * S::kPitch + kk);
+        if (kSwiglu) u[j] = *reinterpret_cast<const float4*>(su + (tx + kTx * j) * S::kPitch + kk);
+      }
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+          acc0[i][j] = fmaf(a[i].x, b[j].x, acc0[i][j]);
+          acc0[i][j] = fmaf(a[i].y, b[j].y, acc0[i][j]);
+          acc0[i][j] = fmaf(a[i].z, b[j].z, acc0[i][j]);
+          acc0[i][j] = fmaf(a[i].w, b[j].w, acc0[i][j]);
+          if (kSwiglu) {
+            acc1[i][j] = fmaf(a[i].x, u[j].x, acc1[i][j]);
+            acc1[i][j] = fmaf(a[i].y, u[j].y, acc1[i][j]);
+            acc1[i][j] = fmaf(a[i].z, u[j].z, acc1[i][j]);
+            acc1[i][j] = fmaf(a[i].w, u[j].w, acc1[i][j]);
+          }
+        }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < TM; ++i) {
+    const int r = r0 + ty + kTy * i;
+    if (r >= te.rows) continue;
+    float* orow = out + static_cast<int64_t>(te.out_row0 + r) * n_out;
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+      const int c = c0 + tx + kTx * j;
+      if (c < n_out) {
+        const float g = acc0[i][j];
+        orow[c] = kSwiglu ? g / (1.0f + expf(-g)) * acc1[i][j] : g;
+      }
+    }
+  }
+}
+
+template <int BM, int BN, int TM, int TN, int BK>
+cudaError_t launch_tile(bool swiglu, const float* A, const float* Wb0, const float* Wb1,
+                        const GemmArgs& g, cudaStream_t st) {
+  const int col_blocks = (g.n_out + BN - 1) / BN;
+  const int64_t blocks = static_cast<int64_t>(col_blocks) * g.max_tiles * (kTileM / BM);
+  if (blocks > INT32_MAX) return cudaErrorInvalidValue;
+  const dim3 grid(static_cast<unsigned>(blocks));
+  const int threads = SimtTile<BM, BN, TM, TN, BK, true>::kThreads;
+  auto* kern = swiglu ? expert_simt_kernel<BM, BN, TM, TN, BK, true>
+                      : expert_simt_kernel<BM, BN, TM, TN, BK, false>;
+  return launch_pdl(kern, grid, dim3(threads), 0, st, 1, A, g.perm, g.k, Wb0, Wb1,
+                    static_cast<const TileEntry*>(g.tiles), g.num_tiles, g.K, g.n_out,
+                    g.b_rows_per_expert, col_blocks, static_cast<float*>(g.out),
+                    static_cast<const int32_t*>(g.status));
 }
 
 }  // namespace
 
 cudaError_t launch_expert_simt(bool swiglu, const float* A, const float* Wb0, const float* Wb1,
-                               const GemmArgs& g, cudaStream_t st) {
+                               const GemmArgs& g, int64_t rows, int num_sms, cudaStream_t st) {
   if (g.max_tiles <= 0) return cudaSuccess;
-  dim3 grid(g.max_tiles, (g.n_out + kCols - 1) / kCols);
-  return launch_pdl(expert_simt_kernel, grid, dim3(kCols), 0, st, 1, swiglu ? 1 : 0, A, Wb0, Wb1,
-                    static_cast<const TileEntry*>(g.tiles), g.num_tiles, g.K, g.n_out,
-                    g.b_rows_per_expert, static_cast<float*>(g.out),
-                    static_cast<const int32_t*>(g.status));
+  // 64 x 64 blocks move half the bytes per FMA of 32 x 32 ones, but only once they fill the GPU
+  // twice over; below that the shorter blocks win by their number.
+  const int64_t big = ((rows + 63) / 64) * ((g.n_out + 63) / 64);
+  return big >= 2 * static_cast<int64_t>(num_sms)
+             ? launch_tile<64, 64, 4, 4, 16>(swiglu, A, Wb0, Wb1, g, st)
+             : launch_tile<32, 32, 4, 2, 32>(swiglu, A, Wb0, Wb1, g, st);
 }
 
 }  // namespace pr2

@@ -102,7 +102,7 @@ cudaError_t launch_route_tc(int mode, const CUtensorMap& tm_h, const CUtensorMap
 struct DispatchArgs {
   const int32_t* idx;
   int64_t T;
-  int k, N, d, esz, n_shared;
+  int k, N, n_shared;
   int32_t* blk_hist;     // [nblk, N] block histograms, scanned in place into block bases
   int32_t* counts;       // [N]
   int32_t* offsets;      // [N+1]
@@ -112,8 +112,6 @@ struct DispatchArgs {
   int32_t* num_tiles;    // [2]: routed M-tiles, shared M-tiles
   TileEntry* stiles1;    // [n_shared * ceil(T/128)] gate/up GEMM of the shared experts
   TileEntry* stiles2;    // same, down GEMM
-  const void* h;
-  void* xperm;           // [T*k, d] permuted copy of h (fp32 path); nullptr: no gather launch
   int32_t* status;
   unsigned int* sync_ctr;  // grid-barrier counter of the fused dispatch (zeroed per call)
   int32_t* ready;          // [max_mtiles] per M-tile counters of the fused GEMM, cleared here
@@ -151,8 +149,7 @@ struct GemmArgs {
   void* out;                 // [rows, n_out]
   int32_t* status;
   // Gathered A (gate/up GEMM of the routed experts): row r of a tile is token perm[r] / k of
-  // `a_src` [T, K] instead of row r of a permuted copy.  Unused when the A operand comes from
-  // the tensor map.
+  // `a_src` [T, K] (bf16) or of the A argument (fp32).  Unused where A has its own rows.
   const void* a_src;
   const int32_t* perm;
   int k;
@@ -174,8 +171,9 @@ struct MlpArgs {
 cudaError_t launch_expert_tc(ExpertKind kind, const CUtensorMap& tm_a, const CUtensorMap& tm_b0,
                              const CUtensorMap& tm_b1, const CUtensorMap& tm_b2,
                              const MlpArgs& a, int num_sms, cudaStream_t st);
+// fp32: rows A[perm[r] / k] when g.perm is set, else A[r]; `rows` = rows over all tiles.
 cudaError_t launch_expert_simt(bool swiglu, const float* A, const float* Wb0, const float* Wb1,
-                               const GemmArgs& g, cudaStream_t st);
+                               const GemmArgs& g, int64_t rows, int num_sms, cudaStream_t st);
 
 // ---- predictive loss gradient (predictor.cu) ---------------------------------------------
 // grad_Wp = (1/T_c) G^T h_old with G = dKL/dz.  bf16: split-K tcgen05 GEMM over tokens into
