@@ -646,7 +646,7 @@ def run_pr2(args, rank, world, local_rank):
         per["layer_replay"].append(el(e[3], e[6]))
         for _, st in (e[2], e[5]):
             per["dispatch"].append(el(st[0], st[1]))
-            # routed gate/up and down run as one launch (plus the shared experts' GEMMs)
+            # routed gate/up and down run as one launch (shared experts included)
             per["expert_gemm"].append(el(st[1], st[3]))
             per["combine"].append(el(st[3], st[4]))
     value = replicas.job_throughput(cfg.T * args.steps, world, total_ms)
@@ -793,11 +793,11 @@ def run_pr2(args, rank, world, local_rank):
 
     # per layer forward: dispatch (one fused cooperative kernel when N % 4 == 0 and the grid is
     # resident, as at every bench shape; else hist + scan + place), the routed grouped GEMMs (one
-    # launch for gate/up and down in bf16, two in fp32; + two for shared experts) and the
+    # launch for gate/up and down in bf16, two in fp32, shared experts included) and the
     # combine; plus one routing kernel per mode
     n_dispatch = 1 if cfg.N % 4 == 0 and cfg.N <= 256 else 3
     n_gemm = 1 if cfg.dtype == "bf16" else 2
-    launches_per_step = 2 + 2 * (n_dispatch + n_gemm + 1 + (2 if cfg.n_shared else 0))
+    launches_per_step = 2 + 2 * (n_dispatch + n_gemm + 1)
     line = dict(metric=METRIC, value=value, unit="tokens/s", n_gpus=world, steps=args.steps,
                 warmup=args.warmup, ms_per_step=total_ms / args.steps, higher_is_better=True,
                 scaling="weak", vs_baseline=None, dtype=cfg.dtype, data="synthetic",

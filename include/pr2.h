@@ -115,10 +115,9 @@ pr2_status pr2_route_replay(const pr2_dims* dims, const void* h, const void* W_r
 typedef struct {
     void* start;         /* before dispatch                                              */
     void* dispatched;    /* after histogram, scan and stable placement                    */
-    void* gate_up_done;  /* after the routed experts' GEMMs (bf16: gate/up and down run as
-                          * one launch) and the shared experts' gate/up GEMM              */
-    void* down_done;     /* after the shared experts' down GEMM (the routed down GEMM on
-                          * the fp32 path)                                               */
+    void* gate_up_done;  /* after the gate/up GEMM (bf16: gate/up and down of every expert
+                          * run as one launch, both events come after it)                 */
+    void* down_done;     /* after the down GEMM                                           */
     void* end;           /* after the gate-weighted combine                              */
 } pr2_stage_events;
 

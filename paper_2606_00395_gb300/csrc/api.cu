@@ -82,14 +82,10 @@ struct Workspace {
   unsigned int* sync_ctr;
   int32_t* ready;
   TileEntry* tiles;
-  TileEntry* stiles1;
-  TileEntry* stiles2;
   int32_t* route_hist;  // per-CTA expert histograms of the rollout routing (pr2_moe_rollout_forward)
-  void* hbuf;
-  void* ybuf;
-  void* hs;
-  void* ys;
-  int nblk, max_tiles, shared_tiles;
+  void* hbuf;  // [T k + n_shared T, m]: routed rows in dispatch order, then the shared experts'
+  void* ybuf;  // [T k + n_shared T, d]
+  int nblk, max_tiles;
   size_t total;
 };
 
@@ -104,34 +100,31 @@ Workspace carve(const pr2_dims& dm, uint8_t* base) {
   const int64_t F = dm.T * dm.k;
   const size_t es = esize(dm);
   w.nblk = static_cast<int>((F + kDispatchChunk - 1) / kDispatchChunk);
-  w.max_tiles = static_cast<int>(F / kTileM + dm.N + 1);
   const int mt_T = static_cast<int>((dm.T + kTileM - 1) / kTileM);
-  w.shared_tiles = dm.n_shared * mt_T;
+  // tiles of at most 128 rows or more
+  w.max_tiles = static_cast<int>(F / kMinTileRows + dm.N + 1) +
+                dm.n_shared * static_cast<int>((dm.T + kMinTileRows - 1) / kMinTileRows);
   w.status = reinterpret_cast<int32_t*>(take(sizeof(int32_t)));
   w.blk_hist = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * (size_t)w.nblk * dm.N));
   w.counts = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * dm.N));
   w.offsets = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * (dm.N + 1)));
   w.perm = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * F));
   w.inv = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * F));
-  w.num_tiles = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * 2));
+  w.num_tiles = reinterpret_cast<int32_t*>(take(sizeof(int32_t)));
   w.sync_ctr = reinterpret_cast<unsigned int*>(take(sizeof(unsigned int)));
   w.ready = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * w.max_tiles));
   w.tiles = reinterpret_cast<TileEntry*>(take(sizeof(TileEntry) * w.max_tiles));
-  w.stiles1 = reinterpret_cast<TileEntry*>(take(sizeof(TileEntry) * (w.shared_tiles + 1)));
-  w.stiles2 = reinterpret_cast<TileEntry*>(take(sizeof(TileEntry) * (w.shared_tiles + 1)));
-
   // fp32: the size that callers plan with includes a permuted copy of h, which no kernel writes
   // (the gate/up GEMMs of both types gather their rows from h)
   if (dm.dtype == PR2_FP32) take(es * F * dm.d);
   // H [Tk, m].  The rollout routing's per-CTA histograms share its first bytes: dispatch reads
   // them before the gate/up GEMM (which waits for dispatch) writes H.
   const size_t hist_bytes = sizeof(int32_t) * (size_t)mt_T * kRouteMaxSplit * dm.N;
-  const size_t h_bytes = es * F * dm.m;
+  const int64_t rows = F + dm.n_shared * dm.T;
+  const size_t h_bytes = es * rows * dm.m;
   w.hbuf = take(h_bytes > hist_bytes ? h_bytes : hist_bytes);
   w.route_hist = static_cast<int32_t*>(w.hbuf);
-  w.ybuf = take(es * F * dm.d);
-  w.hs = take(es * dm.n_shared * dm.T * dm.m);
-  w.ys = take(es * dm.n_shared * dm.T * dm.d);
+  w.ybuf = take(es * rows * dm.d);
   w.total = off;
   return w;
 }
@@ -462,9 +455,11 @@ pr2_status moe_forward_impl(const pr2_dims* dims, const void* h, const int32_t* 
   };
   mark(events ? events->start : nullptr);
 
-  DispatchArgs da{idx,       dm.T,      dm.k,   dm.N,  dm.n_shared, w.blk_hist,  w.counts,
-                  w.offsets, w.perm,    w.inv,  w.tiles, w.num_tiles, w.stiles1, w.stiles2,
-                  status,    w.sync_ctr, dm.dtype == PR2_BF16 ? w.ready : nullptr, kTileM};
+  const int64_t F = dm.T * dm.k;
+  const int tile_rows = dm.dtype == PR2_BF16 ? expert_tile_rows(F, dm.N) : kMinTileRows;
+  DispatchArgs da{idx,    dm.T,    dm.k,        dm.N,    dm.n_shared,  w.blk_hist, w.counts,
+                  w.offsets, w.perm, w.inv,     w.tiles, w.num_tiles, status,     w.sync_ctr,
+                  dm.dtype == PR2_BF16 ? w.ready : nullptr, tile_rows};
   if (err == cudaSuccess)
     err = (rhist != nullptr && dm.dtype == PR2_BF16)
               ? launch_dispatch_from_hist(da, rhist->hist, rhist->split, st)
@@ -472,57 +467,37 @@ pr2_status moe_forward_impl(const pr2_dims* dims, const void* h, const int32_t* 
   mark(events ? events->dispatched : nullptr);
   if (err != cudaSuccess) return PR2_ERR_CUDA;
 
-  const int64_t F = dm.T * dm.k;
-  GemmArgs g1{w.tiles, w.num_tiles, w.max_tiles, dm.d, dm.m, dm.m, w.hbuf, status,
-              h, w.perm, dm.k};  // gathered A
-  GemmArgs g2{w.tiles, w.num_tiles, w.max_tiles, dm.m, dm.d, dm.d, w.ybuf, status,
-              nullptr, nullptr, 0};
-  GemmArgs s1{w.stiles1, w.num_tiles + 1, w.shared_tiles, dm.d, dm.m, dm.m, w.hs, status,
-              nullptr, nullptr, 0};
-  GemmArgs s2{w.stiles2, w.num_tiles + 1, w.shared_tiles, dm.m, dm.d, dm.d, w.ys, status,
-              nullptr, nullptr, 0};
   if (dm.dtype == PR2_BF16) {
-    CUtensorMap b1g, b1u, a2, b2, sa1, sb1g, sb1u, sa2, sb2;
-    bool ok = make_tmap_bf16(&b1g, W_gate, dm.d, (uint64_t)dm.N * dm.m, 64, 128) &&
-              make_tmap_bf16(&b1u, W_up, dm.d, (uint64_t)dm.N * dm.m, 64, 128) &&
-              make_tmap_bf16(&a2, w.hbuf, dm.m, F, 64, kTileM) &&
-              make_tmap_bf16(&b2, W_down, dm.m, (uint64_t)dm.N * dm.d, 64, 256);
+    ExpertMaps tm;
+    bool ok = make_tmap_bf16(&tm.gate, W_gate, dm.d, (uint64_t)dm.N * dm.m, 64, 128) &&
+              make_tmap_bf16(&tm.up, W_up, dm.d, (uint64_t)dm.N * dm.m, 64, 128) &&
+              make_tmap_bf16(&tm.down, W_down, dm.m, (uint64_t)dm.N * dm.d, 64, 128);
     if (ok && dm.n_shared > 0) {
-      ok = make_tmap_bf16(&sa1, h, dm.d, dm.T, 64, kTileM) &&
-           make_tmap_bf16(&sb1g, Ws_gate, dm.d, (uint64_t)dm.n_shared * dm.m, 64, 128) &&
-           make_tmap_bf16(&sb1u, Ws_up, dm.d, (uint64_t)dm.n_shared * dm.m, 64, 128) &&
-           make_tmap_bf16(&sa2, w.hs, dm.m, (uint64_t)dm.n_shared * dm.T, 64, kTileM) &&
-           make_tmap_bf16(&sb2, Ws_down, dm.m, (uint64_t)dm.n_shared * dm.d, 64, 256);
+      ok = make_tmap_bf16(&tm.s_gate, Ws_gate, dm.d, (uint64_t)dm.n_shared * dm.m, 64, 128) &&
+           make_tmap_bf16(&tm.s_up, Ws_up, dm.d, (uint64_t)dm.n_shared * dm.m, 64, 128) &&
+           make_tmap_bf16(&tm.s_down, Ws_down, dm.m, (uint64_t)dm.n_shared * dm.d, 64, 128);
+    } else {
+      tm.s_gate = tm.gate;
+      tm.s_up = tm.up;
+      tm.s_down = tm.down;
     }
     if (!ok) return PR2_ERR_CUDA;
-    // routed experts: gate/up then down in one cooperative launch
-    MlpArgs routed{{g1, g2}, w.ready};
-    err = launch_expert_tc(kExpertFused, a2, b1g, b1u, b2, routed, num_sms, st);
-    if (err == cudaSuccess && dm.n_shared > 0) {
-      MlpArgs sh1{{s1, s1}, nullptr};
-      err = launch_expert_tc(kExpertGateUpTma, sa1, sb1g, sb1u, sb1g, sh1, num_sms, st);
-    }
+    const MlpArgs ma{w.tiles, w.num_tiles, w.max_tiles, w.ready, h,      w.perm, dm.k,
+                     dm.N,    dm.d,        dm.m,        w.hbuf,  w.ybuf, status};
+    err = launch_expert_tc(tm, ma, tile_rows, num_sms, st);
     mark(events ? events->gate_up_done : nullptr);
-    if (err == cudaSuccess && dm.n_shared > 0) {
-      MlpArgs sh2{{s2, s2}, nullptr};
-      err = launch_expert_tc(kExpertDown, sa2, sb2, sb2, sb2, sh2, num_sms, st);
-    }
     mark(events ? events->down_done : nullptr);
   } else {
-    const int64_t FS = dm.T * dm.n_shared;  // rows of the shared experts
-    err = launch_expert_simt(true, static_cast<const float*>(h), static_cast<const float*>(W_gate),
-                             static_cast<const float*>(W_up), g1, F, num_sms, st);
-    if (err == cudaSuccess && dm.n_shared > 0)
-      err = launch_expert_simt(true, static_cast<const float*>(h),
-                               static_cast<const float*>(Ws_gate),
-                               static_cast<const float*>(Ws_up), s1, FS, num_sms, st);
+    auto f32 = [](const void* p) { return static_cast<const float*>(p); };
+    const int64_t rows = F + dm.n_shared * dm.T;
+    SimtArgs g{w.tiles, w.num_tiles, w.max_tiles, dm.d, dm.m, dm.k, dm.N, f32(h), f32(W_gate),
+               f32(W_up), f32(Ws_gate), f32(Ws_up), w.perm, static_cast<float*>(w.hbuf), status};
+    err = launch_expert_simt(true, g, rows, num_sms, st);
     mark(events ? events->gate_up_done : nullptr);
-    if (err == cudaSuccess)
-      err = launch_expert_simt(false, static_cast<const float*>(w.hbuf),
-                               static_cast<const float*>(W_down), nullptr, g2, F, num_sms, st);
-    if (err == cudaSuccess && dm.n_shared > 0)
-      err = launch_expert_simt(false, static_cast<const float*>(w.hs),
-                               static_cast<const float*>(Ws_down), nullptr, s2, FS, num_sms, st);
+    SimtArgs g2{w.tiles, w.num_tiles, w.max_tiles, dm.m, dm.d, dm.k, dm.N, f32(w.hbuf),
+                f32(W_down), nullptr, f32(Ws_down), nullptr, w.perm, static_cast<float*>(w.ybuf),
+                status};
+    if (err == cudaSuccess) err = launch_expert_simt(false, g2, rows, num_sms, st);
     mark(events ? events->down_done : nullptr);
   }
   if (err != cudaSuccess) return PR2_ERR_CUDA;
@@ -538,7 +513,8 @@ pr2_status moe_forward_impl(const pr2_dims* dims, const void* h, const int32_t* 
     if (s != PR2_OK) return s;
   }
 
-  CombineArgs ca{w.ybuf, dm.n_shared > 0 ? w.ys : nullptr, w.inv, gates, dm.T, dm.k, dm.d,
+  const void* ys = dm.n_shared > 0 ? static_cast<uint8_t*>(w.ybuf) + esize(dm) * F * dm.d : nullptr;
+  CombineArgs ca{w.ybuf, ys, w.inv, gates, dm.T, dm.k, dm.d,
                  dm.n_shared, dm.dtype == PR2_BF16 ? 1 : 0, out, residual, status};
   err = launch_combine(ca, num_sms, st);
   mark(events ? events->end : nullptr);

@@ -5,8 +5,8 @@
 //   1. hist   - one block per 256 slots: validate each slot (expert in [0,N), not repeated in
 //               its token) and count per expert in shared memory -> blk_hist[b][e].
 //   2. scan   - one block: per expert an exclusive scan over blocks (in place), the expert
-//               totals (counts), their exclusive scan (offsets), the M-tile table of the
-//               grouped GEMM, and the static tile tables of the shared experts.
+//               totals (counts), their exclusive scan (offsets) and the tile table of the
+//               grouped GEMMs.
 //   3. place  - one block per 256 slots again: per-warp counts via __match_any_sync, a scan
 //               over the 8 warps, then rank = popc(lanes below with the same expert):
 //               perm[offsets[e] + r] = f, inv[f] = its position (-1 for an invalid slot).
@@ -14,8 +14,8 @@
 // Steps 1-3 normally run as one cooperative launch (dispatch_fused_kernel): every block counts
 // its slots, one bounded grid barrier, then each block derives the expert totals, its own
 // per-expert bases and the expert offsets from the whole block histogram (identical in every
-// block), block 0 writes counts, offsets and the tile tables (and clears the grouped GEMM's
-// per-M-tile readiness counters), and every block places its slots.  Shapes whose grid cannot
+// block), block 0 writes counts, offsets and the tile table (and clears the grouped GEMM's
+// per-tile readiness counters), and every block places its slots.  Shapes whose grid cannot
 // be resident at once use the three kernels above.
 // Combine (the sums of Eqs. pr2_old_output / pr2_output):
 //   out[t, :] = sum_s gates[t,s] * Y[inv[t*k+s], :] + sum_j Ys[j, t, :], fp32 accumulation,
@@ -93,58 +93,50 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* sh, int* total) 
 }
 
 // The grouped GEMM's tile table: each expert's rows split into ceil(rows / tile_rows) tiles of
-// near-equal size (entry i belongs to the expert whose tile range contains i; its per-tile
-// readiness counter is cleared) and the static tile tables of the shared experts
-// (every token: gate/up reads rows of h, down rows of Hs), from the experts' row offsets ex_off
-// and first tiles ex_tile (N + 1 entries each, in shared memory); num_tiles[0..1] = their
-// lengths.  Called by every thread of one block.
-__device__ void write_tile_tables(int N, int64_t T, int n_shared, int tile_rows,
-                                  const int* ex_off, const int* ex_tile,
-                                  TileEntry* __restrict__ tiles,
-                                  int32_t* __restrict__ num_tiles,
-                                  TileEntry* __restrict__ stiles1,
-                                  TileEntry* __restrict__ stiles2, int32_t* __restrict__ ready) {
+// near-equal size, a multiple of 16 rows but for the last (entry i belongs to the expert whose
+// tile range contains i; its per-tile readiness counter is cleared), then the shared experts'
+// tiles (expert N + j: every token, rows T k + j T + t of H and Y), from the experts' row offsets
+// ex_off and first tiles ex_tile (N + 1 entries each, in shared memory); num_tiles[0] = its
+// length.  Called by every thread of one block.
+__device__ void write_tile_table(int N, int64_t T, int k, int n_shared, int tile_rows,
+                                 const int* ex_off, const int* ex_tile,
+                                 TileEntry* __restrict__ tiles, int32_t* __restrict__ num_tiles,
+                                 int32_t* __restrict__ ready) {
   const int tid = threadIdx.x;
-  const int all_tiles = ex_tile[N];
-  const int mt_T = static_cast<int>((T + kTileM - 1) / kTileM);
-  if (tid == 0) {
-    num_tiles[0] = all_tiles;
-    num_tiles[1] = n_shared * mt_T;
-  }
-  for (int i = tid; i < all_tiles; i += blockDim.x) {
-    int lo = 0, hi = N - 1;
-    while (lo < hi) {  // last expert with ex_tile[ex] <= i
-      const int mid = (lo + hi + 1) >> 1;
-      if (ex_tile[mid] <= i) lo = mid; else hi = mid - 1;
+  const int routed = ex_tile[N];
+  const int per_shared = static_cast<int>((T + tile_rows - 1) / tile_rows);
+  const int all = routed + n_shared * per_shared;
+  if (tid == 0) num_tiles[0] = all;
+  for (int i = tid; i < all; i += blockDim.x) {
+    if (ready != nullptr) ready[i] = 0;
+    if (i < routed) {
+      int lo = 0, hi = N - 1;
+      while (lo < hi) {  // last expert with ex_tile[ex] <= i
+        const int mid = (lo + hi + 1) >> 1;
+        if (ex_tile[mid] <= i) lo = mid; else hi = mid - 1;
+      }
+      const int j = i - ex_tile[lo];
+      const int nch = ex_tile[lo + 1] - ex_tile[lo];
+      const int c = ex_off[lo + 1] - ex_off[lo];
+      const int sz = ((c + nch - 1) / nch + 15) & ~15;  // (nch - 1) sz < c: no tile is empty
+      const int r0 = ex_off[lo] + j * sz;
+      const int left = ex_off[lo + 1] - r0;
+      tiles[i] = TileEntry{lo, r0, left < sz ? left : sz, r0};
+    } else {
+      const int j = (i - routed) / per_shared, t0 = (i - routed) % per_shared * tile_rows;
+      const int rows = T - t0 < tile_rows ? static_cast<int>(T - t0) : tile_rows;
+      tiles[i] = TileEntry{N + j, t0, rows, static_cast<int>(T * k + j * T) + t0};
     }
-    // the expert's c rows split into nch = ceil(c / tile_rows) tiles of near-equal size
-    const int j = i - ex_tile[lo];
-    const int nch = ex_tile[lo + 1] - ex_tile[lo];
-    const int c = ex_off[lo + 1] - ex_off[lo];
-    const int sz = (c + nch - 1) / nch;
-    const int r0 = ex_off[lo] + j * sz;
-    const int left = ex_off[lo + 1] - r0;
-    tiles[i] = TileEntry{lo, r0, left < sz ? left : sz, r0};
-    if (ready != nullptr) ready[i] = 0;  // per M-tile counter of the fused expert GEMM
-  }
-  for (int i = tid; i < n_shared * mt_T; i += blockDim.x) {
-    const int j = i / mt_T, m = i - j * mt_T;
-    const int r0 = m * kTileM;
-    const int rows = (T - r0) < kTileM ? static_cast<int>(T - r0) : kTileM;
-    const int o0 = static_cast<int>(j * T) + r0;
-    stiles1[i] = TileEntry{j, r0, rows, o0};
-    stiles2[i] = TileEntry{j, o0, rows, o0};
   }
 }
 
 // One block of 1024 threads = G groups of N_pad threads: thread (g, e) owns expert e over the
 // block range of group g, so the per-expert scans over blocks run G-way parallel.
 __global__ void __launch_bounds__(1024)
-    scan_kernel(int32_t* __restrict__ blk_hist, int nblk, int N, int64_t T, int n_shared,
+    scan_kernel(int32_t* __restrict__ blk_hist, int nblk, int N, int64_t T, int k, int n_shared,
                 int tile_rows,
                 int32_t* __restrict__ counts, int32_t* __restrict__ offsets,
                 TileEntry* __restrict__ tiles, int32_t* __restrict__ num_tiles,
-                TileEntry* __restrict__ stiles1, TileEntry* __restrict__ stiles2,
                 int32_t* __restrict__ ready) {
   __shared__ int sh[32];
   __shared__ int part[1024];  // [G][N_pad] partial sums, then their exclusive scan over g
@@ -214,8 +206,7 @@ __global__ void __launch_bounds__(1024)
       }
     }
   }
-  write_tile_tables(N, T, n_shared, tile_rows, ex_off, ex_tile, tiles, num_tiles, stiles1,
-                    stiles2, ready);
+  write_tile_table(N, T, k, n_shared, tile_rows, ex_off, ex_tile, tiles, num_tiles, ready);
 }
 
 __global__ void __launch_bounds__(kDispatchChunk)
@@ -288,8 +279,7 @@ __global__ void __launch_bounds__(kDispatchChunk)
                           int n_shared, int tile_rows, int32_t* blk_hist, int32_t* __restrict__ counts,
                           int32_t* __restrict__ offsets, int32_t* __restrict__ perm,
                           int32_t* __restrict__ inv, TileEntry* __restrict__ tiles,
-                          int32_t* __restrict__ num_tiles, TileEntry* __restrict__ stiles1,
-                          TileEntry* __restrict__ stiles2, unsigned int* sync_ctr,
+                          int32_t* __restrict__ num_tiles, unsigned int* sync_ctr,
                           int32_t* status, int32_t* __restrict__ ready) {
   extern __shared__ int dsm[];
   int* wcnt = dsm;                   // [kWarps][N] per-warp counts, then per-warp bases
@@ -400,8 +390,7 @@ __global__ void __launch_bounds__(kDispatchChunk)
       offsets[tid] = off;
     }
     if (tid == 0) offsets[N] = all_rows;
-    write_tile_tables(N, T, n_shared, tile_rows, ex_off, ex_tile, tiles, num_tiles, stiles1,
-                      stiles2, ready);
+    write_tile_table(N, T, k, n_shared, tile_rows, ex_off, ex_tile, tiles, num_tiles, ready);
   }
   // ---- 3. stable placement: per-warp bases, then ranks within the warp
   for (int x = tid; x < N; x += blockDim.x) {
@@ -439,7 +428,6 @@ __global__ void __launch_bounds__(kHistBlock)
                          int split, int32_t* __restrict__ counts, int32_t* __restrict__ offsets,
                          int32_t* __restrict__ perm, int32_t* __restrict__ inv,
                          TileEntry* __restrict__ tiles, int32_t* __restrict__ num_tiles,
-                         TileEntry* __restrict__ stiles1, TileEntry* __restrict__ stiles2,
                          int32_t* __restrict__ ready) {
   extern __shared__ int dsm[];
   int* wcnt = dsm;                     // [kHistWarps][N] per-warp counts, then per-warp bases
@@ -524,8 +512,7 @@ __global__ void __launch_bounds__(kHistBlock)
       offsets[tid] = off;
     }
     if (tid == 0) offsets[N] = all_rows;
-    write_tile_tables(N, T, n_shared, tile_rows, ex_off, ex_tile, tiles, num_tiles, stiles1,
-                      stiles2, ready);
+    write_tile_table(N, T, k, n_shared, tile_rows, ex_off, ex_tile, tiles, num_tiles, ready);
   }
   // ---- stable placement: per-warp bases, then ranks within the warp
   for (int x = tid; x < N; x += kHistBlock) {
@@ -840,7 +827,7 @@ cudaError_t launch_dispatch(const DispatchArgs& a, int num_sms, cudaStream_t st)
     cfg.numAttrs = 1;
     err = cudaLaunchKernelEx(&cfg, dispatch_fused_kernel, a.idx, F, a.k, a.N, a.T, a.n_shared,
                              a.tile_rows, a.blk_hist, a.counts, a.offsets, a.perm, a.inv, a.tiles,
-                             a.num_tiles, a.stiles1, a.stiles2, a.sync_ctr, a.status, a.ready);
+                             a.num_tiles, a.sync_ctr, a.status, a.ready);
     if (err != cudaSuccess) return err;
   } else {
     if (nblk > 0) {
@@ -848,9 +835,8 @@ cudaError_t launch_dispatch(const DispatchArgs& a, int num_sms, cudaStream_t st)
                        a.N, a.blk_hist, a.status);
       if (err != cudaSuccess) return err;
     }
-    err = launch_pdl(scan_kernel, dim3(1), dim3(1024), 0, st, 1, a.blk_hist, nblk, a.N, a.T,
-                     a.n_shared, a.tile_rows, a.counts, a.offsets, a.tiles, a.num_tiles, a.stiles1,
-                     a.stiles2, a.ready);
+    err = launch_pdl(scan_kernel, dim3(1), dim3(1024), 0, st, 1, a.blk_hist, nblk, a.N, a.T, a.k,
+                     a.n_shared, a.tile_rows, a.counts, a.offsets, a.tiles, a.num_tiles, a.ready);
     if (err != cudaSuccess) return err;
     if (nblk > 0) {
       err = launch_pdl(place_kernel, dim3(nblk), dim3(kDispatchChunk), 0, st, 1, a.idx, F, a.k,
@@ -873,8 +859,7 @@ cudaError_t launch_dispatch_from_hist(const DispatchArgs& a, const int32_t* hist
   if (err != cudaSuccess) return err;
   return launch_pdl(dispatch_hist_kernel, dim3(tiles_r), dim3(kHistBlock), smem, st, 1, a.idx,
                     a.T, a.k, a.N, a.n_shared, a.tile_rows, hist, tiles_r * split, split,
-                    a.counts, a.offsets, a.perm, a.inv, a.tiles, a.num_tiles, a.stiles1,
-                    a.stiles2, a.ready);
+                    a.counts, a.offsets, a.perm, a.inv, a.tiles, a.num_tiles, a.ready);
 }
 
 cudaError_t launch_combine(const CombineArgs& a, int num_sms, cudaStream_t st) {

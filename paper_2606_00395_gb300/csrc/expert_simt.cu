@@ -30,12 +30,6 @@ __device__ __forceinline__ void cp_async_4(uint32_t smem_dst, const void* src, u
                "r"(src_bytes)
                : "memory");
 }
-__device__ __forceinline__ void cp_async_16(uint32_t smem_dst, const void* src,
-                                            uint32_t src_bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_dst), "l"(src),
-               "r"(src_bytes)
-               : "memory");
-}
 
 template <int BM, int BN, int TM, int TN, int BK, bool kSwiglu>
 struct SimtTile {
@@ -52,21 +46,23 @@ struct SimtTile {
 
 template <int BM, int BN, int TM, int TN, int BK, bool kSwiglu>
 __global__ void __launch_bounds__((SimtTile<BM, BN, TM, TN, BK, kSwiglu>::kThreads))
-    expert_simt_kernel(const float* __restrict__ A, const int32_t* __restrict__ perm, int k,
-                       const float* __restrict__ W0, const float* __restrict__ W1,
-                       const TileEntry* __restrict__ tiles, const int32_t* __restrict__ num_tiles,
-                       int K, int n_out, int b_rows, int col_blocks, float* __restrict__ out,
-                       const int32_t* status) {
+    expert_simt_kernel(SimtArgs g, int col_blocks) {
   using S = SimtTile<BM, BN, TM, TN, BK, kSwiglu>;
   __shared__ __align__(16) float smem[kStages * S::kStageFloats];
-  constexpr int kSub = kTileM / BM;  // row blocks of one M-tile
+  constexpr int kSub = kMinTileRows / BM;  // row blocks of one M-tile
   pdl_wait();
   pdl_trigger();
   // mt < max_tiles by the grid; a dispatch that timed out leaves the table unwritten
   const int row_block = static_cast<int>(blockIdx.x) / col_blocks;
   const int mt = row_block / kSub;
-  if (status_timed_out(status) || mt >= *num_tiles) return;
-  const TileEntry te = tiles[mt];
+  if (status_timed_out(g.status) || mt >= *g.num_tiles) return;
+  const TileEntry te = g.tiles[mt];
+  const int K = g.K, n_out = g.n_out;
+  const float* __restrict__ A = g.A;
+  const bool shared = te.expert >= g.N;
+  const float* __restrict__ W0 = shared ? g.S0 : g.W0;
+  const float* __restrict__ W1 = shared ? g.S1 : g.W1;
+  const int64_t wrow0 = static_cast<int64_t>(shared ? te.expert - g.N : te.expert) * n_out;
   const int r0 = (row_block % kSub) * BM;
   if (r0 >= te.rows) return;
   const int c0 = (static_cast<int>(blockIdx.x) % col_blocks) * BN;
@@ -83,14 +79,15 @@ __global__ void __launch_bounds__((SimtTile<BM, BN, TM, TN, BK, kSwiglu>::kThrea
     src[i] = A;
     if (row < BM) {
       if (r0 + row < te.rows) {
-        const int p = te.a_row0 + r0 + row;
-        src[i] = A + static_cast<int64_t>(perm != nullptr ? perm[p] / k : p) * K + kc;
+        // gate/up: the token at this place (shared experts: the token itself); down: its H row
+        const int p = (kSwiglu ? te.a_row0 : te.out_row0) + r0 + row;
+        src[i] = A + static_cast<int64_t>(kSwiglu && !shared ? g.perm[p] / g.k : p) * K + kc;
         on |= 1u << i;
       }
     } else {
       const int c = c0 + (row - BM) % BN;
       if (c < n_out) {
-        src[i] = (row - BM < BN ? W0 : W1) + (static_cast<int64_t>(te.expert) * b_rows + c) * K + kc;
+        src[i] = (row - BM < BN ? W0 : W1) + (wrow0 + c) * K + kc;
         on |= 1u << i;
       }
     }
@@ -179,45 +176,41 @@ __global__ void __launch_bounds__((SimtTile<BM, BN, TM, TN, BK, kSwiglu>::kThrea
   for (int i = 0; i < TM; ++i) {
     const int r = r0 + ty + kTy * i;
     if (r >= te.rows) continue;
-    float* orow = out + static_cast<int64_t>(te.out_row0 + r) * n_out;
+    float* orow = g.out + static_cast<int64_t>(te.out_row0 + r) * n_out;
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
       const int c = c0 + tx + kTx * j;
       if (c < n_out) {
-        const float g = acc0[i][j];
-        orow[c] = kSwiglu ? g / (1.0f + expf(-g)) * acc1[i][j] : g;
+        const float v = acc0[i][j];
+        orow[c] = kSwiglu ? v / (1.0f + expf(-v)) * acc1[i][j] : v;
       }
     }
   }
 }
 
 template <int BM, int BN, int TM, int TN, int BK>
-cudaError_t launch_tile(bool swiglu, const float* A, const float* Wb0, const float* Wb1,
-                        const GemmArgs& g, cudaStream_t st) {
+cudaError_t launch_tile(bool swiglu, const SimtArgs& g, cudaStream_t st) {
   const int col_blocks = (g.n_out + BN - 1) / BN;
-  const int64_t blocks = static_cast<int64_t>(col_blocks) * g.max_tiles * (kTileM / BM);
+  const int64_t blocks = static_cast<int64_t>(col_blocks) * g.max_tiles * (kMinTileRows / BM);
   if (blocks > INT32_MAX) return cudaErrorInvalidValue;
   const dim3 grid(static_cast<unsigned>(blocks));
   const int threads = SimtTile<BM, BN, TM, TN, BK, true>::kThreads;
   auto* kern = swiglu ? expert_simt_kernel<BM, BN, TM, TN, BK, true>
                       : expert_simt_kernel<BM, BN, TM, TN, BK, false>;
-  return launch_pdl(kern, grid, dim3(threads), 0, st, 1, A, g.perm, g.k, Wb0, Wb1,
-                    static_cast<const TileEntry*>(g.tiles), g.num_tiles, g.K, g.n_out,
-                    g.b_rows_per_expert, col_blocks, static_cast<float*>(g.out),
-                    static_cast<const int32_t*>(g.status));
+  return launch_pdl(kern, grid, dim3(threads), 0, st, 1, g, col_blocks);
 }
 
 }  // namespace
 
-cudaError_t launch_expert_simt(bool swiglu, const float* A, const float* Wb0, const float* Wb1,
-                               const GemmArgs& g, int64_t rows, int num_sms, cudaStream_t st) {
+cudaError_t launch_expert_simt(bool swiglu, const SimtArgs& g, int64_t rows, int num_sms,
+                               cudaStream_t st) {
   if (g.max_tiles <= 0) return cudaSuccess;
   // 64 x 64 blocks move half the bytes per FMA of 32 x 32 ones, but only once they fill the GPU
   // twice over; below that the shorter blocks win by their number.
   const int64_t big = ((rows + 63) / 64) * ((g.n_out + 63) / 64);
   return big >= 2 * static_cast<int64_t>(num_sms)
-             ? launch_tile<64, 64, 4, 4, 16>(swiglu, A, Wb0, Wb1, g, st)
-             : launch_tile<32, 32, 4, 2, 32>(swiglu, A, Wb0, Wb1, g, st);
+             ? launch_tile<64, 64, 4, 4, 16>(swiglu, g, st)
+             : launch_tile<32, 32, 4, 2, 32>(swiglu, g, st);
 }
 
 }  // namespace pr2

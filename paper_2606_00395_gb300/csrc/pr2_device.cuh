@@ -75,6 +75,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
+// Whether the phase has completed, without waiting (try_wait may suspend the thread).
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // Wait for the phase with the given parity to complete.  Returns false (after recording the
 // timeout) if it did not within `limit_ns`, or as soon as another role raised `abort_flag`.
 static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
@@ -145,6 +158,12 @@ __device__ __forceinline__ void tma_load_2d_hint(void* smem_dst, const void* tma
 // written through the generic proxy: the thread that acquires the barrier executes
 // fence.proxy.async before a tcgen05.mma (async proxy) reads it.
 // ------------------------------------------------------------------------------------------
+__device__ __forceinline__ void cp_async_16(uint32_t smem_dst, const void* src,
+                                            uint32_t src_bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_dst), "l"(src),
+               "r"(src_bytes)
+               : "memory");
+}
 // With an L2 eviction-priority hint (a createpolicy value).
 __device__ __forceinline__ void cp_async_16_hint(uint32_t smem_dst, const void* src,
                                                  uint32_t src_bytes, uint64_t policy) {
@@ -167,13 +186,20 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-// Acquire load at GPU scope (pairs with a writer's __threadfence() + atomic), and the proxy
-// fence that then makes the observed generic-proxy writes to global memory visible to TMA loads
-// (async proxy) issued by this thread.
+// Acquire load at GPU scope (pairs with a writer's __threadfence() + atomic), and an acquire load
+// / release store of a shared-memory word at CTA scope.
 __device__ __forceinline__ int ld_acquire_gpu(const int* p) {
   int v;
   asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
+}
+__device__ __forceinline__ int ld_acquire_cta(const int* shared) {
+  int v;
+  asm volatile("ld.acquire.cta.shared.b32 %0, [%1];" : "=r"(v) : "r"(smem_u32(shared)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_release_cta(int* shared, int v) {
+  asm volatile("st.release.cta.shared.b32 [%0], %1;" ::"r"(smem_u32(shared)), "r"(v) : "memory");
 }
 // Whether an earlier kernel of the call recorded PR2_STATUS_TIMEOUT in the status word (read
 // after pdl_wait).  The kernels that consume dispatch's tables (grouped GEMMs, combine) then do
@@ -182,14 +208,15 @@ __device__ __forceinline__ bool status_timed_out(const int32_t* status) {
   if (status == nullptr) return false;
   return (*reinterpret_cast<const volatile int32_t*>(status) & PR2_STATUS_TIMEOUT) != 0;
 }
-__device__ __forceinline__ void fence_proxy_async_global() {
-  asm volatile("fence.proxy.async.global;" ::: "memory");
+__device__ __forceinline__ void st_global_v4(void* p, const uint32_t (&w)[4]) {
+  asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(w[0]), "r"(w[1]),
+               "r"(w[2]), "r"(w[3])
+               : "memory");
 }
-
-// One 32-byte store (a full L2 sector) of eight 32-bit words; `p` must be 32-byte aligned.
-__device__ __forceinline__ void st_global_v8(void* p, const uint32_t (&w)[8]) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(w[0]),
-               "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+__device__ __forceinline__ void ld_shared_v4(uint32_t smem, uint32_t (&w)[4]) {
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+               : "r"(smem)
                : "memory");
 }
 
@@ -240,6 +267,30 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr) {
   desc |= static_cast<uint64_t>(1u) << 46;
   desc |= static_cast<uint64_t>(2u) << 61;
   return desc;
+}
+
+// The same descriptor from the tile's 16-byte address units (smem address >> 4): lo is
+// umma_lo(address) plus any offset in those units (32 bytes of K = 2).
+__device__ __forceinline__ uint32_t umma_lo(uint32_t smem_addr) {
+  return ((smem_addr & 0x3FFFFu) >> 4) | (1u << 16);
+}
+__device__ __forceinline__ uint64_t umma_desc_lo(uint32_t lo) {
+  return (static_cast<uint64_t>((1024u >> 4) | (1u << 14) | (2u << 29)) << 32) | lo;
+}
+
+// True in one lane of a converged warp.  The MMA loops run warp-uniformly and issue under this
+// predicate: with descriptors and barriers known to be the same in every lane the compiler keeps
+// them in uniform registers, and an MMA issues in ~35 clk instead of the ~65 clk it takes from a
+// loop that a single thread runs behind `if (lane == 0)` (8 MMAs of N = 16 and one commit: 555
+// instead of 803 clk).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r != 0;
 }
 
 // Descriptor of an MN-major operand tile with the 128-byte swizzle: each 128-B row holds 64
@@ -311,6 +362,41 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[16]) {
                : "memory");
 }
 
+// 16 lanes x 16 columns in the fragment layout of an m16n8 accumulator: for column group i (8
+// columns), thread t holds in r[4 i .. 4 i + 3] lane t / 4, columns 8 i + 2 (t % 4) and the next,
+// then the same of lane t / 4 + 8.  Valid after tmem_wait_ld8().
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld8(uint32_t (&a)[8], uint32_t (&b)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]),
+                 "+r"(a[6]), "+r"(a[7]), "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]),
+                 "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7])
+               :
+               : "memory");
+}
+__device__ __forceinline__ void reg_fence8(uint32_t (&a)[8], uint32_t (&b)[8]) {
+  asm volatile(""
+               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]),
+                 "+r"(a[6]), "+r"(a[7]), "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]),
+                 "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7]));
+}
+// Four 8 x 8 bf16 matrices held as fragments (row t / 4, columns 2 (t % 4) and the next in the low
+// and high half of a register), stored transposed: thread 8 i + k gives the 16-byte address that
+// column k of matrix i goes to.
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t smem, uint32_t a, uint32_t b, uint32_t c,
+                                                  uint32_t d) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(smem),
+               "r"(a), "r"(b), "r"(c), "r"(d)
+               : "memory");
+}
+
 // Pins a second register group behind an already executed tmem_wait_ld().
 __device__ __forceinline__ void reg_fence(uint32_t (&r)[16]) {
   asm volatile(""
@@ -323,6 +409,20 @@ __device__ __forceinline__ void reg_fence(uint32_t (&r)[16]) {
 // Barrier `id` (1-15) over `count` threads (a multiple of 32) of this CTA.
 __device__ __forceinline__ void named_bar_sync(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
+// The same barrier, returning whether `pred` held in every thread of it.
+__device__ __forceinline__ bool named_bar_and(int id, int count, bool pred) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %3, 0;\n\t"
+      "barrier.cta.red.and.pred q, %1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(id), "r"(count), "r"(pred ? 1u : 0u)
+      : "memory");
+  return r != 0;
 }
 
 // Thread-block clusters and distributed shared memory.

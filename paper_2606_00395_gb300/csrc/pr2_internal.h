@@ -37,13 +37,13 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// One M-tile of a grouped GEMM: rows [a_row0, a_row0 + rows) of the A operand, multiplied by
-// the weights of `expert`, written to rows [out_row0, out_row0 + rows) of the output.
+// One tile of a grouped GEMM: `rows` rows multiplied by the weights of `expert` (see MlpArgs).
 struct TileEntry {
   int32_t expert, a_row0, rows, out_row0;
 };
 
-constexpr int kTileM = 128;         // rows per M-tile (one tcgen05 M=128 accumulator)
+constexpr int kTileM = 128;         // tokens of a routing tile (one tcgen05 M=128 accumulator)
+constexpr int kMinTileRows = 128;   // least tile_rows of a grouped GEMM (fp32: its only value)
 constexpr int kDispatchChunk = 256; // flat slots per dispatch block (8 warps x 32 lanes)
 constexpr int kMaxTopK = 8;         // slots kept by the tensor-core routing epilogue
 constexpr int kMaxTopKSimt = 32;    // slots of the fp32 SIMT routing kernel
@@ -108,15 +108,13 @@ struct DispatchArgs {
   int32_t* offsets;      // [N+1]
   int32_t* perm;         // [T*k]
   int32_t* inv;          // [T*k]
-  TileEntry* tiles;      // [max_mtiles]
-  int32_t* num_tiles;    // [2]: routed M-tiles, shared M-tiles
-  TileEntry* stiles1;    // [n_shared * ceil(T/128)] gate/up GEMM of the shared experts
-  TileEntry* stiles2;    // same, down GEMM
+  TileEntry* tiles;      // [max_tiles]: the routed experts' tiles, then the shared experts'
+  int32_t* num_tiles;    // [1]
   int32_t* status;
   unsigned int* sync_ctr;  // grid-barrier counter of the fused dispatch (zeroed per call)
-  int32_t* ready;          // [max_mtiles] per M-tile counters of the fused GEMM, cleared here
+  int32_t* ready;          // [max_tiles] per-tile counters of the bf16 GEMM, cleared here
                            // (nullable)
-  int tile_rows;           // most rows of one routed tile (an expert's rows are split evenly)
+  int tile_rows;           // most rows of one tile (an expert's rows are split evenly)
 };
 cudaError_t launch_dispatch(const DispatchArgs& a, int num_sms, cudaStream_t st);
 // Dispatch of a route the routing kernel just wrote (every slot valid), from the per-CTA
@@ -139,41 +137,48 @@ struct CombineArgs {
 cudaError_t launch_combine(const CombineArgs& a, int num_sms, cudaStream_t st);
 
 // ---- grouped expert GEMMs (expert_tc.cu, expert_simt.cu) -----------------------------------
-struct GemmArgs {
+// Tiles of the table: routed experts e < N (rows a_row0.. of the permutation), then shared
+// experts N + j (tokens a_row0..); rows of H and Y from out_row0 (routed: a_row0; shared expert
+// j's token t: T k + j T + t).
+// bf16: gate/up with the SwiGLU epilogue into H, then down into Y, in one cooperative launch.
+struct MlpArgs {
   const TileEntry* tiles;
   const int32_t* num_tiles;  // device count of valid entries in `tiles`
   int max_tiles;             // host bound on that count
-  int K;                     // reduction length
-  int n_out;                 // output columns
-  int b_rows_per_expert;     // rows of one expert's weight matrix (m for gate/up, d for down)
-  void* out;                 // [rows, n_out]
+  int32_t* ready;            // per tile count of finished gate/up epilogue warps, zero on entry
+                             // (dispatch clears it)
+  const void* h;             // [T, d]
+  const int32_t* perm;       // row r of a routed tile is token perm[r] / k of h
+  int k, N, d, m;
+  void* H;                   // [T k + n_shared T, m]
+  void* Y;                   // [T k + n_shared T, d]
   int32_t* status;
-  // Gathered A (gate/up GEMM of the routed experts): row r of a tile is token perm[r] / k of
-  // `a_src` [T, K] (bf16) or of the A argument (fp32).  Unused where A has its own rows.
-  const void* a_src;
+};
+// Weight maps, boxes of 128 rows (s_*: shared experts; copies of
+// the routed maps when there are none).
+struct ExpertMaps {
+  CUtensorMap gate, up, down, s_gate, s_up, s_down;
+};
+// Most rows of one tile of a launch over `rows` routed rows and N experts (128 or 256).
+int expert_tile_rows(int64_t rows, int N);
+cudaError_t launch_expert_tc(const ExpertMaps& tm, const MlpArgs& a, int tile_rows, int num_sms,
+                             cudaStream_t st);
+
+// fp32, one GEMM: gate/up (W0 = gate, W1 = up, A = h) or down (W0 = down, A = H).
+struct SimtArgs {
+  const TileEntry* tiles;
+  const int32_t* num_tiles;
+  int max_tiles;
+  int K, n_out;              // reduction length, output columns (= weight rows of an expert)
+  int k, N;
+  const float *A, *W0, *W1, *S0, *S1;  // S: the shared experts' weights (nullable)
   const int32_t* perm;
-  int k;
+  float* out;
+  const int32_t* status;
 };
-// Launch kinds of the tcgen05 grouped GEMM (expert_tc.cu).  Phase 0 is a gate/up GEMM with the
-// SwiGLU epilogue (weights tm_b0 = gate, tm_b1 = up), phase 1 a down GEMM (weights tm_b2).
-enum ExpertKind : int {
-  kExpertGateUpTma = 1,     // phase 0, A rows from tm_a (shared experts: rows of h)
-  kExpertDown = 2,          // phase 1, A rows from tm_a
-  kExpertFused = 3,         // phase 0, A rows gathered from p[0].a_src through p[0].perm,
-                            // then phase 1 (A = p[0].out through tm_a), in one cooperative
-                            // launch (the routed experts)
-};
-struct MlpArgs {
-  GemmArgs p[2];     // arguments of phase 0 and phase 1 (only the launched phases are read)
-  int32_t* ready;    // kExpertFused: per M-tile count of finished gate/up epilogue warps,
-                     // zero on entry (dispatch clears it)
-};
-cudaError_t launch_expert_tc(ExpertKind kind, const CUtensorMap& tm_a, const CUtensorMap& tm_b0,
-                             const CUtensorMap& tm_b1, const CUtensorMap& tm_b2,
-                             const MlpArgs& a, int num_sms, cudaStream_t st);
-// fp32: rows A[perm[r] / k] when g.perm is set, else A[r]; `rows` = rows over all tiles.
-cudaError_t launch_expert_simt(bool swiglu, const float* A, const float* Wb0, const float* Wb1,
-                               const GemmArgs& g, int64_t rows, int num_sms, cudaStream_t st);
+// `rows` = rows over all tiles.
+cudaError_t launch_expert_simt(bool swiglu, const SimtArgs& g, int64_t rows, int num_sms,
+                               cudaStream_t st);
 
 // ---- predictive loss gradient (predictor.cu) ---------------------------------------------
 // grad_Wp = (1/T_c) G^T h_old with G = dKL/dz.  bf16: split-K tcgen05 GEMM over tokens into
