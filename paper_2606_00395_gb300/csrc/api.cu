@@ -541,14 +541,19 @@ pr2_status pr2_moe_forward(const pr2_dims* dims, const void* h, const int32_t* i
                           stream);
 }
 
-pr2_status pr2_moe_rollout_forward(const pr2_dims* dims, const void* h, const void* W_router,
-                                   const void* W_pred, int32_t* idx, float* gates,
-                                   float* logits_old, int64_t* near_tie, const void* W_gate,
-                                   const void* W_up, const void* W_down, const void* Ws_gate,
-                                   const void* Ws_up, const void* Ws_down, void* out,
-                                   int32_t* counts, int32_t* perm, void* workspace,
-                                   size_t ws_bytes, int32_t* status_dev,
-                                   const pr2_stage_events* events, void* stream) {
+}  // extern "C"
+
+namespace pr2 {
+namespace {
+
+// The rollout layer of pr2_moe_rollout_forward; `residual` as in moe_forward_impl.
+pr2_status rollout_impl(const pr2_dims* dims, const void* h, const void* W_router,
+                        const void* W_pred, int32_t* idx, float* gates, float* logits_old,
+                        int64_t* near_tie, const void* W_gate, const void* W_up,
+                        const void* W_down, const void* Ws_gate, const void* Ws_up,
+                        const void* Ws_down, void* out, const void* residual, int32_t* counts,
+                        int32_t* perm, void* workspace, size_t ws_bytes, int32_t* status_dev,
+                        const pr2_stage_events* events, void* stream) {
   pr2_status s = check_dims(dims);
   if (s != PR2_OK) return s;
   const pr2_dims& dm = *dims;
@@ -568,7 +573,7 @@ pr2_status pr2_moe_rollout_forward(const pr2_dims* dims, const void* h, const vo
                      status_dev, stream);
     if (s != PR2_OK) return s;
     return moe_forward_impl(dims, h, idx, gates, W_gate, W_up, W_down, Ws_gate, Ws_up, Ws_down,
-                            out, nullptr, counts, perm, workspace, ws_bytes, status_dev, events,
+                            out, residual, counts, perm, workspace, ws_bytes, status_dev, events,
                             stream);
   }
   const Workspace w = carve(dm, static_cast<uint8_t*>(workspace));
@@ -578,8 +583,26 @@ pr2_status pr2_moe_rollout_forward(const pr2_dims* dims, const void* h, const vo
   if (s != PR2_OK) return s;
   const RouteHist rh{w.route_hist, split};
   return moe_forward_impl(dims, h, idx, gates, W_gate, W_up, W_down, Ws_gate, Ws_up, Ws_down,
-                          out, nullptr, counts, perm, workspace, ws_bytes, status_dev, events,
+                          out, residual, counts, perm, workspace, ws_bytes, status_dev, events,
                           stream, nullptr, &rh);
+}
+
+}  // namespace
+}  // namespace pr2
+
+extern "C" {
+
+pr2_status pr2_moe_rollout_forward(const pr2_dims* dims, const void* h, const void* W_router,
+                                   const void* W_pred, int32_t* idx, float* gates,
+                                   float* logits_old, int64_t* near_tie, const void* W_gate,
+                                   const void* W_up, const void* W_down, const void* Ws_gate,
+                                   const void* Ws_up, const void* Ws_down, void* out,
+                                   int32_t* counts, int32_t* perm, void* workspace,
+                                   size_t ws_bytes, int32_t* status_dev,
+                                   const pr2_stage_events* events, void* stream) {
+  return rollout_impl(dims, h, W_router, W_pred, idx, gates, logits_old, near_tie, W_gate, W_up,
+                      W_down, Ws_gate, Ws_up, Ws_down, out, nullptr, counts, perm, workspace,
+                      ws_bytes, status_dev, events, stream);
 }
 
 pr2_status pr2_moe_replay_forward(const pr2_dims* dims, const void* h, const void* W_router,
@@ -632,13 +655,11 @@ pr2_status pr2_rollout_layers(const pr2_dims* dims, int32_t L, void* h, const vo
     int32_t* idx_l = idx + (size_t)l * dm.T * dm.k;
     float* gates_l = gates + (size_t)l * dm.T * dm.k;
     float* logits_l = logits_old ? logits_old + (size_t)l * dm.T * dm.N : nullptr;
-    s = pr2_route_predict(&dl, h, base(W_router, l * r_sz), base(W_pred, l * r_sz), idx_l,
-                          gates_l, logits_l, near_tie, status_dev, stream);
-    if (s != PR2_OK) return s;
-    s = moe_forward_impl(&dl, h, idx_l, gates_l, base(W_gate, l * gu_sz), base(W_up, l * gu_sz),
-                         base(W_down, l * gu_sz), base(Ws_gate, l * sgu_sz),
-                         base(Ws_up, l * sgu_sz), base(Ws_down, l * sgu_sz), h, h, nullptr,
-                         nullptr, workspace, ws_bytes, status_dev, nullptr, stream);
+    s = rollout_impl(&dl, h, base(W_router, l * r_sz), base(W_pred, l * r_sz), idx_l, gates_l,
+                     logits_l, near_tie, base(W_gate, l * gu_sz), base(W_up, l * gu_sz),
+                     base(W_down, l * gu_sz), base(Ws_gate, l * sgu_sz), base(Ws_up, l * sgu_sz),
+                     base(Ws_down, l * sgu_sz), h, h, nullptr, nullptr, workspace, ws_bytes,
+                     status_dev, nullptr, stream);
     if (s != PR2_OK) return s;
   }
   return finish(cudaSuccess, dm.flags, status_dev, static_cast<cudaStream_t>(stream));
