@@ -126,16 +126,28 @@ def declared_symbols() -> list:
     return sorted(set(re.findall(r"\b(pr2_[a-z_0-9]+)\s*\(", hdr)))
 
 
+# The small entry points are a few microseconds of GPU work behind one launch, so the call itself
+# counts: pointers and the stream go through as plain integers (the argtypes make them void *),
+# and the current stream is asked of torch's C layer without building a Stream object (a
+# feature-cache call took 9.0 us of host time before and takes 4.6, six tracking calls 67 and 38).
+
 def _p(t: Optional[torch.Tensor]):
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _s(stream) -> ctypes.c_void_p:
+_get_device = getattr(torch._C, "_cuda_getDevice", None)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_cuda_ready = False
+
+
+def _s(stream) -> int:
+    global _cuda_ready
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        if _cuda_ready:
+            return _raw_stream(_get_device())
+        stream = torch.cuda.current_stream()  # initialises CUDA, or raises
+        _cuda_ready = _get_device is not None and _raw_stream is not None
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def check(code: int, where: str = "pr2") -> None:
@@ -172,7 +184,7 @@ def pr2_moe_forward(dm: Dims, h, idx, gates, W_gate, W_up, W_down, Ws_gate, Ws_u
     return load().pr2_moe_forward(ctypes.byref(dm), _p(h), _p(idx), _p(gates), _p(W_gate),
                                   _p(W_up), _p(W_down), _p(Ws_gate), _p(Ws_up), _p(Ws_down),
                                   _p(out), _p(counts), _p(perm), _p(workspace),
-                                  ctypes.c_size_t(ws_bytes), _p(status),
+                                  ws_bytes, _p(status),
                                   None if events is None else ctypes.byref(events), _s(stream))
 
 
@@ -187,7 +199,7 @@ def pr2_moe_rollout_forward(dm: Dims, h, W_router, W_pred, idx, gates, logits_ol
     return load().pr2_moe_rollout_forward(
         ctypes.byref(dm), _p(h), _p(W_router), _p(W_pred), _p(idx), _p(gates), _p(logits_old),
         _p(near_tie), _p(W_gate), _p(W_up), _p(W_down), _p(Ws_gate), _p(Ws_up), _p(Ws_down),
-        _p(out), _p(counts), _p(perm), _p(workspace), ctypes.c_size_t(ws_bytes), _p(status),
+        _p(out), _p(counts), _p(perm), _p(workspace), ws_bytes, _p(status),
         None if events is None else ctypes.byref(events), _s(stream))
 
 
@@ -202,7 +214,7 @@ def pr2_moe_replay_forward(dm: Dims, h, W_router, idx, gates, probs, W_gate, W_u
     return load().pr2_moe_replay_forward(
         ctypes.byref(dm), _p(h), _p(W_router), _p(idx), _p(gates), _p(probs), _p(W_gate),
         _p(W_up), _p(W_down), _p(Ws_gate), _p(Ws_up), _p(Ws_down), _p(out), _p(counts), _p(perm),
-        _p(workspace), ctypes.c_size_t(ws_bytes), _p(status),
+        _p(workspace), ws_bytes, _p(status),
         None if events is None else ctypes.byref(events), _s(stream))
 
 
@@ -223,7 +235,7 @@ def pr2_predictor_loss(dm: Dims, h_old, p_old, W_pred, rho, loss, grad, pos=None
     T_rho = int(rho.shape[0]) if rho is not None else 0
     return load().pr2_predictor_loss(ctypes.byref(dm), _p(h_old), _p(p_old), _p(W_pred), _p(rho),
                                      T_rho, _p(pos), _p(loss), _p(kl_tok), _p(grad),
-                                     _p(workspace), ctypes.c_size_t(ws_bytes), _p(status),
+                                     _p(workspace), ws_bytes, _p(status),
                                      _s(stream))
 
 
@@ -249,7 +261,7 @@ def pr2_rollout_layers(dm: Dims, L: int, h, W_router, W_pred, W_gate, W_up, W_do
     return load().pr2_rollout_layers(ctypes.byref(dm), int(L), _p(h), _p(W_router), _p(W_pred),
                                      _p(W_gate), _p(W_up), _p(W_down), _p(Ws_gate), _p(Ws_up),
                                      _p(Ws_down), _p(idx), _p(gates), _p(logits_old),
-                                     _p(near_tie), _p(workspace), ctypes.c_size_t(ws_bytes),
+                                     _p(near_tie), _p(workspace), ws_bytes,
                                      _p(status), _s(stream))
 
 
