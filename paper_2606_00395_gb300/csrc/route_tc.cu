@@ -18,15 +18,23 @@
 // Warp roles: warp 0 = TMA producer, warp 1 = TMEM owner and MMA issuer, warps 2..5 = epilogue.
 // With S > 1 the partials are reduce-scattered by rows through distributed shared memory: CTA q
 // receives rows [q 128/S, (q+1) 128/S) of every CTA's partial, stored [source][column/4][row][4]
-// so that each warp store moves contiguous bytes; the four epilogue warps then sum the S copies
-// once, in source order (deterministic), walking consecutive 16-byte words so that no two lanes
-// of a warp hit one bank.  Each row is then finished by S consecutive threads, thread `part` owning experts
-// [part N/S, (part+1) N/S); with S = 1 one thread finishes its row straight from TMEM.  A thread
-// reduces its experts to a max, a sum of exp(z - max) and (predict) its top-16 by 64-bit keys
-// (orderable z bits, inverted expert index: z descending, ties to the lower expert), built by
-// bitonic sorting 16 experts at a time and merging, in one pass with a running (online) softmax
-// sum; the S threads of a row then combine max and sum (sum_q s_q exp(m_q - max), fixed shuffle
-// order) and merge their lists by shuffles.
+// so that each warp store moves contiguous bytes; rows beyond the batch are not moved.  Two ways
+// to finish the rows:
+//  - by warps (predict with 64 < N <= 128, S >= 4): all six warps sum the S copies once, in source
+//    order (deterministic), into rows of shared memory, and each then finishes whole rows, up to
+//    six at a time: a lane holds four experts, and the top k + 1 come out one by one by warp maxima
+//    (redux.sync) over orderable 32-bit values.  Sum and rows of a T = 256 predict call: 4.4 us by
+//    threads, 2.9 us by warps (3.7 with five shuffles instead of redux.sync); eight experts per
+//    lane (N = 256, 64 rows per CTA) 24 us where threads take 11.
+//  - by threads (everything else): the four epilogue warps sum the S copies in place, walking
+//    consecutive 16-byte words so that no two lanes of a warp hit one bank.  Each row is then
+//    finished by S consecutive threads, thread `part` owning experts [part N/S, (part+1) N/S);
+//    with S = 1 one thread finishes its row straight from TMEM.  A thread reduces its experts to
+//    a max, a sum of exp(z - max) and (predict) its top-16 by 64-bit keys (orderable z bits,
+//    inverted expert index: z descending, ties to the lower expert), built by bitonic sorting 16
+//    experts at a time and merging, in one pass with a running (online) softmax sum; the S
+//    threads of a row then combine max and sum (sum_q s_q exp(m_q - max), fixed shuffle order)
+//    and merge their lists by shuffles.
 // Selection is on z in fp32 (softmax is monotone, so the order equals the order of rho_hat).
 #include <float.h>
 
@@ -78,6 +86,21 @@ __host__ __device__ inline RouteSmemLayout route_layout(int N, bool predict, boo
 // Bytes of the reduce-scatter buffer, [S][NB/S/4][128][4] fp32, placed over the pipeline
 // stages once every CTA of the cluster has finished its K blocks.
 __host__ __device__ inline int route_recv_bytes(int b_rows) { return b_rows * kTileM * 4; }
+
+// Whether predict rows are finished by warps: 16 or 32 rows per CTA of more than 64 experts (calls
+// with N = 128: T = 600, S = 8 13.0 us by threads, 11.1 by warps; T = 4001, S = 4 16.4 / 16.15;
+// T = 8192, S = 2 21.8 / 25.2; N = 64, T = 4096, S = 4 11.1 / 11.7).
+__host__ __device__ inline bool route_by_warps(int N, int split) {
+  return N > 64 && N <= 128 && split >= 4;
+}
+// The rows that they move into row order at a time, behind the received copies: the largest power
+// of two (at most the CTA's rows) that fits.
+__host__ __device__ inline int route_finish_rows(const RouteSmemLayout& L, int split) {
+  const int row = (L.b_rows / 4 + 1) * 16;
+  int rc = 1;
+  while (rc < kTileM / split && route_recv_bytes(L.b_rows) + 2 * rc * row <= L.bar_offset) rc *= 2;
+  return rc;
+}
 
 __host__ __device__ inline uint32_t tmem_cols_for(int cols) {
   uint32_t c = 32;
@@ -169,6 +192,118 @@ __device__ __forceinline__ bool predict_write(const uint64_t (&key)[16], float m
   return (a.k < a.N) && (pk - pk1 < (float)PR2_NEAR_TIE_GAP);
 }
 
+// Orderable bits of z (z descending = bits descending), at least 1: 0 marks a removed expert.
+__device__ __forceinline__ uint32_t order_bits(float z) {
+  const uint32_t u = __float_as_uint(z);
+  const uint32_t ord = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+  return ord > 1u ? ord : 1u;
+}
+__device__ __forceinline__ float order_value(uint32_t ord) {
+  return __uint_as_float((ord & 0x80000000u) ? (ord & 0x7fffffffu) : ~ord);
+}
+__device__ __forceinline__ float warp_add(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Finishes kRB predict rows by one warp (N <= 128).  Row j: [p_old | b] of 2 N floats at rows[j] in
+// shared memory, token t[j] (live[j]: inside the batch).  Lane l holds experts 4 l .. 4 l + 3,
+// sorted once; the top k + 1 then come out one by one, the lane whose head equals the warp's
+// maximum giving it (the lowest such lane: z descending, ties to the lower expert).  Writes p_old,
+// idx, gates (divided by their sum under PR2_F_NORMALIZE_TOPK), counts the experts into `hist`
+// (with `count`) and returns the number of rows with rho_hat_(k) - rho_hat_(k+1) <
+// PR2_NEAR_TIE_GAP, always on the unnormalised probabilities.
+template <int kRB>
+__device__ __forceinline__ int finish_predict_rows(const float4* const (&rows)[kRB],
+                                                   const int64_t (&t)[kRB],
+                                                   const bool (&live)[kRB], const RouteTcArgs& a,
+                                                   bool count, int (&hist)[kMaxExperts]) {
+  const int lane = threadIdx.x & 31;
+  const int n4 = a.N / 4;
+  uint32_t key[kRB][4];
+  uint32_t ids[kRB];  // the lane's experts in the order of its keys, 4 bits each
+  float mx[kRB], sum[kRB], my_z[kRB];
+  int my_e[kRB];
+#pragma unroll
+  for (int j = 0; j < kRB; ++j) {
+    float z[4];
+    if (lane < n4) {
+      const float4 p = rows[j][lane], b = rows[j][n4 + lane];
+      if (a.logits_or_probs != nullptr && live[j])
+        reinterpret_cast<float4*>(a.logits_or_probs + t[j] * a.N)[lane] = p;
+      z[0] = p.x + b.x;
+      z[1] = p.y + b.y;
+      z[2] = p.z + b.z;
+      z[3] = p.w + b.w;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) key[j][q] = order_bits(z[q]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        z[q] = -INFINITY;
+        key[j][q] = 0u;
+      }
+    }
+    uint32_t id[4] = {0u, 1u, 2u, 3u};
+    // odd-even transposition: neighbours swap only when out of order, so equal values keep theirs
+#pragma unroll
+    for (int ph = 0; ph < 4; ++ph)
+#pragma unroll
+      for (int q = ph & 1; q + 1 < 4; q += 2) {
+        const bool sw = key[j][q + 1] > key[j][q];
+        const uint32_t k0 = key[j][q], i0 = id[q];
+        key[j][q] = sw ? key[j][q + 1] : k0;
+        key[j][q + 1] = sw ? k0 : key[j][q + 1];
+        id[q] = sw ? id[q + 1] : i0;
+        id[q + 1] = sw ? i0 : id[q + 1];
+      }
+    ids[j] = id[0] | id[1] << 4 | id[2] << 8 | id[3] << 12;
+    mx[j] = fmaxf(order_value(__reduce_max_sync(0xffffffffu, key[j][0])), -FLT_MAX);
+    sum[j] = 0.f;
+    if (lane < n4)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) sum[j] += expf(z[q] - mx[j]);
+    my_z[j] = 0.f;
+    my_e[j] = 0;
+  }
+  const int rounds = a.k < a.N ? a.k + 1 : a.k;
+  for (int r = 0; r < rounds; ++r) {
+#pragma unroll
+    for (int j = 0; j < kRB; ++j) {
+      const uint32_t m = __reduce_max_sync(0xffffffffu, key[j][0]);
+      const unsigned has = __ballot_sync(0xffffffffu, key[j][0] == m);
+      const int owner = __ffs(has) - 1;
+      const int e = __shfl_sync(0xffffffffu, lane * 4 + static_cast<int>(ids[j] & 15u), owner);
+      if (lane == r) {
+        my_z[j] = order_value(m);
+        my_e[j] = e;
+      }
+      if (lane == owner) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) key[j][q] = key[j][q + 1];
+        key[j][3] = 0u;
+        ids[j] >>= 4;
+      }
+    }
+  }
+  int ties = 0;
+#pragma unroll
+  for (int j = 0; j < kRB; ++j) {
+    const float pr = expf(my_z[j] - mx[j]) * (1.0f / warp_add(sum[j]));
+    const float sk = a.norm ? warp_add(lane < a.k ? pr : 0.f) : 0.f;
+    if (live[j] && lane < a.k) {
+      a.idx_out[t[j] * a.k + lane] = my_e[j];
+      a.gates[t[j] * a.k + lane] = a.norm ? pr * (1.0f / sk) : pr;
+      if (count) atomicAdd(&hist[my_e[j]], 1);
+    }
+    const float pk = __shfl_sync(0xffffffffu, pr, a.k - 1);
+    const float pk1 = __shfl_sync(0xffffffffu, pr, a.k);  // k <= 8
+    ties += (live[j] && a.k < a.N && pk - pk1 < (float)PR2_NEAR_TIE_GAP) ? 1 : 0;
+  }
+  return ties;
+}
+
 template <int kMode, int split>
 __global__ void __launch_bounds__(kThreads, 1)
     route_tc_kernel(const __grid_constant__ CUtensorMap tm_h,
@@ -203,6 +338,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // row then meet in the CTA that finishes it, through distributed shared memory, and are not
   // summed.  Otherwise the cluster splits K and the S partial rows are summed.
   const bool psplit = predict && L.passes == 2 && split == 2;
+  const bool by_warps = predict && route_by_warps(N, split);
   const int KBper = psplit ? a.d / kBK : (a.d / kBK) / split;
   const int kb0 = psplit ? 0 : rank * KBper, kb1 = kb0 + KBper;
   const int npass = psplit ? 1 : L.passes;  // passes this CTA streams
@@ -328,9 +464,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   // predict: experts of the rows this CTA finishes, for the dispatch that follows
   __shared__ int hist_s[kMaxExperts];
   const bool count = predict && a.hist != nullptr;
-  if (count && epi) {
+  if (count && epi) {  // (split > 1: the cluster barriers below order it before the counting)
     for (int e = threadIdx.x - 64; e < N; e += 128) hist_s[e] = 0;
-    named_bar_sync(1, 128);
+    if (split == 1) named_bar_sync(1, 128);
   }
   const int q = warp & 3;
   const int row = q * 32 + lane;  // TMEM lane of this thread
@@ -411,12 +547,17 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int off4 = psplit ? L.pass_rows / 4 : nb4;
       const uint32_t rbase =
           mapa_shared(smem_u32(recv_w + (rank * off4) * R + drow), dst);
-      for (int c0 = 0; c0 < acc_cols; c0 += 32) {
+      // rows beyond the batch are not moved (a decode batch fills a few rows of its tile); a
+      // warp of such rows skips its loads too
+      const bool in_batch = static_cast<int64_t>(t0) + row < a.T;
+      const int cols = static_cast<int64_t>(t0) + q * 32 < a.T ? acc_cols : 0;
+      for (int c0 = 0; c0 < cols; c0 += 32) {
         uint32_t r0[16], r1[16];
         tmem_ld16(trow + c0, r0);
         tmem_ld16(trow + c0 + 16, r1);
         tmem_wait_ld(r0);
         reg_fence(r1);
+        if (!in_batch) continue;
 #pragma unroll
         for (int j = 0; j < 4; ++j)
           st_cluster_v4(rbase + static_cast<uint32_t>(((c0 / 4 + j) * R) * 16), r0[4 * j],
@@ -430,7 +571,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     cluster_sync();  // every partial row has landed
-    if (epi && !psplit) {
+    if (epi && !psplit && !by_warps) {
       // Sum the S received copies of this CTA's rows once, in source order, into source 0's
       // slots: consecutive threads take consecutive 16-byte words (no bank conflicts), so the
       // finishing threads then read one value per column instead of S strided ones.
@@ -468,9 +609,59 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   };
 
+  if (split >= 4 && by_warps) {
+    // every thread of the CTA is past the cluster barrier: all six warps sum and finish
+    const int rc = route_finish_rows(L, split);
+    const int pitch4 = nb4 + 1;  // 16-byte words of a row: odd, so 8 rows take 8 bank groups
+    float4* rm = reinterpret_cast<float4*>(smem) + nb4 * kTileM;
+    const int64_t tr = static_cast<int64_t>(t0) + static_cast<int64_t>(rank) * R;
+    int ties = 0;
+    for (int rb = 0; rb < R && tr + rb < a.T; rb += rc) {
+      for (int i = threadIdx.x; i < nb4 * rc; i += kThreads) {
+        const int row_i = i % rc, at = i / rc * R + rb + row_i;
+        float4 v = recv[at];
+#pragma unroll
+        for (int src = 1; src < split; ++src) {
+          const float4 w = recv[src * nb4 * R + at];
+          v.x += w.x;
+          v.y += w.y;
+          v.z += w.z;
+          v.w += w.w;
+        }
+        rm[row_i * pitch4 + i / rc] = v;
+      }
+      __syncthreads();
+      if (*abort_flag == 0) {
+        // a warp's rows interleave; the six warps take the rows at hand in one round
+        constexpr int kRB = split == 4 ? 6 : 3;
+        for (int r = warp * kRB; r < rc && tr + rb + r < a.T; r += (kThreads / 32) * kRB) {
+          const float4* rows[kRB];
+          int64_t ts[kRB];
+          bool lv[kRB];
+#pragma unroll
+          for (int j = 0; j < kRB; ++j) {
+            lv[j] = r + j < rc && tr + rb + r + j < a.T;
+            rows[j] = rm + (lv[j] ? r + j : r) * pitch4;
+            ts[j] = tr + rb + r + j;
+          }
+          ties += finish_predict_rows<kRB>(rows, ts, lv, a, count, hist_s);
+        }
+      }
+      if (rb + rc < R) __syncthreads();  // the rows are read before the next ones take their place
+    }
+    if (lane == 0 && ties != 0 && a.near_tie != nullptr)
+      atomicAdd(reinterpret_cast<unsigned long long*>(a.near_tie),
+                static_cast<unsigned long long>(ties));
+    if (count) {  // every row of this CTA counted: publish its histogram row (zeros included)
+      __syncthreads();
+      int32_t* hrow = a.hist + static_cast<int64_t>(blockIdx.x) * N;
+      for (int e = threadIdx.x; e < N; e += kThreads) hrow[e] = hist_s[e];
+    }
+    if (epi) tc_fence_before();
+  }
   // One pass over this thread's experts, 16 at a time: running max m and sum of exp(z - m),
   // (predict) the top-16 keys, (replay) the z of the cached slots.
-  if (epi && !loss) {
+  if (epi && !loss && !by_warps) {
     bool tie = false;
     float m = -FLT_MAX, sum = 0.f;
     uint64_t top[16];
@@ -546,7 +737,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (have && live && part == 0) {
         tie = predict_write(top, mx, inv_s, t, a);
         if (count)
-          for (int j = 0; j < k; ++j) atomicAdd(&hist_s[key_e(top[j])], 1);
+#pragma unroll
+          for (int j = 0; j < kMaxTopK; ++j)
+            if (j < k) atomicAdd(&hist_s[key_e(top[j])], 1);
       }
     } else if (!loss) {
       // Each valid slot's z is held by the one thread owning its expert; the others hold 0.
@@ -919,6 +1112,7 @@ int route_split(int T, int N, int d, int mode, int num_sms) {
   if (route_recv_bytes(L.b_rows) > L.stages * L.stage_bytes) return 1;
   for (int s = kMaxSplit; s > 1; s >>= 1) {
     if (N % s != 0 || (N / s) % 16 != 0 || KB % s != 0 || tiles * s > num_sms) continue;
+    if (mode == kModePredict && route_by_warps(N, s) && route_finish_rows(L, s) < 2) continue;
     if (max_active_clusters(mode, s, N) < tiles) continue;  // must fit in one wave
     return s;
   }
