@@ -163,7 +163,7 @@ pr2_status route_common(const pr2_dims* dims, bool predict, const void* h, const
   if (dm.dtype == PR2_FP32) {
     err = launch_route_simt(dm, predict, static_cast<const float*>(h),
                             static_cast<const float*>(W), static_cast<const float*>(Wp), idx_in,
-                            idx_out, gates, aux, near_tie, status_dev, st);
+                            idx_out, gates, aux, near_tie, status_dev, late_wait, st);
   } else {
     if (dm.T > (int64_t{1} << 30)) return PR2_ERR_UNSUPPORTED;
     const int num_sms = num_sms_of_current_device();
@@ -502,14 +502,13 @@ pr2_status moe_forward_impl(const pr2_dims* dims, const void* h, const int32_t* 
   }
   if (err != cudaSuccess) return PR2_ERR_CUDA;
   if (replay != nullptr) {
-    // Its inputs (h, the router, the route) are complete before the GEMMs start, so on the
-    // tensor-core path its CTAs take the SMs the GEMM's last CTAs free and wait for the GEMMs
-    // only before exiting; the combine launched behind it then sees both.
+    // Its inputs (h, the router, the route) are complete before the GEMMs start, so its CTAs take
+    // the SMs the GEMM's last CTAs free and wait for the GEMMs only before exiting; the combine
+    // launched behind it then sees both.
     pr2_dims dr = dm;
     dr.flags &= ~PR2_F_SYNC_STATUS;
     s = route_common(&dr, false, h, replay->W_router, nullptr, idx, nullptr,
-                     const_cast<float*>(gates), replay->probs, nullptr, status, stream,
-                     dm.dtype == PR2_BF16);
+                     const_cast<float*>(gates), replay->probs, nullptr, status, stream, true);
     if (s != PR2_OK) return s;
   }
 

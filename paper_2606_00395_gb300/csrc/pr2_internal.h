@@ -55,7 +55,7 @@ constexpr int kRouteMaxSplit = 8;   // most CTAs splitting one routing tile (his
 cudaError_t launch_route_simt(const pr2_dims& dm, bool predict, const float* h, const float* W,
                               const float* Wp, const int32_t* idx_in, int32_t* idx_out,
                               float* gates, float* logits_or_probs, int64_t* near_tie,
-                              int32_t* status, cudaStream_t st);
+                              int32_t* status, bool late_wait, cudaStream_t st);
 
 // Modes of the tensor-core routing kernel (route_tc.cu).
 enum RouteMode : int {
