@@ -15,8 +15,9 @@
 // its slots, one bounded grid barrier, then each block derives the expert totals, its own
 // per-expert bases and the expert offsets from the whole block histogram (identical in every
 // block), block 0 writes counts, offsets and the tile table (and clears the grouped GEMM's
-// per-tile readiness counters), and every block places its slots.  Shapes whose grid cannot
-// be resident at once use the three kernels above.
+// per-tile readiness counters), and every block places its slots.  Batches of up to 1024 slots run
+// all of it in one block (dispatch_small_kernel).  Shapes whose grid cannot be
+// resident at once use the three kernels above.
 // Combine (the sums of Eqs. pr2_old_output / pr2_output):
 //   out[t, :] = sum_s gates[t,s] * Y[inv[t*k+s], :] + sum_j Ys[j, t, :], fp32 accumulation,
 //   plus, when given, a residual row r[t, :] (the multi-layer loop's h_l; may alias out).
@@ -64,7 +65,8 @@ __global__ void __launch_bounds__(kDispatchChunk)
   for (int e = threadIdx.x; e < N; e += blockDim.x) out[e] = hist[e];
 }
 
-// Exclusive block-wide scan of one int per thread (blockDim.x == 1024).
+// Exclusive block-wide scan of one int per thread (a block of kW warps).
+template <int kW>
 __device__ __forceinline__ int block_exclusive_scan(int v, int* sh, int* total) {
   const int tid = threadIdx.x;
   const int lane = tid & 31, w = tid >> 5;
@@ -77,17 +79,17 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* sh, int* total) 
   if (lane == 31) sh[w] = x;
   __syncthreads();
   if (w == 0) {
-    int s = sh[lane];
+    int s = lane < kW ? sh[lane] : 0;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, s, o);
       if (lane >= o) s += y;
     }
-    sh[lane] = s;  // inclusive warp totals
+    if (lane < kW) sh[lane] = s;  // inclusive warp totals
   }
   __syncthreads();
   const int incl = x + (w > 0 ? sh[w - 1] : 0);
-  *total = sh[31];
+  *total = sh[kW - 1];
   __syncthreads();
   return incl - v;
 }
@@ -177,9 +179,9 @@ __global__ void __launch_bounds__(1024)
   }
   __syncthreads();
   int all_rows, all_tiles;
-  const int off = block_exclusive_scan(tid < N ? total : 0, sh, &all_rows);
+  const int off = block_exclusive_scan<32>(tid < N ? total : 0, sh, &all_rows);
   const int ntile_e = tid < N ? (total + tile_rows - 1) / tile_rows : 0;
-  const int tstart = block_exclusive_scan(ntile_e, sh, &all_tiles);
+  const int tstart = block_exclusive_scan<32>(ntile_e, sh, &all_tiles);
   if (tid < N) {
     offsets[tid] = off;
     ex_off[tid] = off;
@@ -246,44 +248,112 @@ __global__ void __launch_bounds__(kDispatchChunk)
   }
 }
 
-// Exclusive scan of one int per thread over a 256-thread block (8 warps).
-__device__ __forceinline__ int block256_exclusive_scan(int v, int* sh, int* total) {
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  int x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) sh[w] = x;
+// Hist, scan and place of at most kSmallSlots slots in one block, a slot per thread: no grid
+// barrier, so neither a counter to clear nor a cooperative launch, and the launch starts behind
+// the kernel before it.  Thread (part, x) sums and then rewrites expert x's counts over its share
+// of the 32 groups of 32 slots.
+constexpr int kSmallSlots = 1024;
+constexpr int kSmallGroups = kSmallSlots / 32;
+
+__global__ void __launch_bounds__(kSmallSlots)
+    dispatch_small_kernel(const int32_t* __restrict__ idx, int F, int k, int N, int64_t T,
+                          int n_shared, int tile_rows, int32_t* __restrict__ counts,
+                          int32_t* __restrict__ offsets, int32_t* __restrict__ perm,
+                          int32_t* __restrict__ inv, TileEntry* __restrict__ tiles,
+                          int32_t* __restrict__ num_tiles, int32_t* status,
+                          int32_t* __restrict__ ready) {
+  extern __shared__ int dsm[];
+  int* gcnt = dsm;                        // [kSmallGroups][N] counts, then positions
+  int* ex_off = gcnt + kSmallGroups * N;  // [N+1]
+  int* ex_tile = ex_off + N + 1;          // [N+1]
+  __shared__ int part[1024];
+  __shared__ int sh[32];
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  for (int i = tid; i < kSmallGroups * N; i += 1024) gcnt[i] = 0;
+  pdl_wait();
+  pdl_trigger();
   __syncthreads();
-  if (w == 0) {
-    int s = lane < kWarps ? sh[lane] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, s, o);
-      if (lane >= o) s += y;
+  int e = -1;
+  if (tid < F && !slot_valid(idx, tid, k, N, &e) && status != nullptr)
+    atomicOr(status, PR2_STATUS_BAD_INDEX);
+  const unsigned same = __match_any_sync(0xffffffffu, e);
+  if (e >= 0 && lane == __ffs(same) - 1) gcnt[w * N + e] = __popc(same);
+  __syncthreads();
+  int n_pad = 32;
+  while (n_pad < N) n_pad <<= 1;
+  const int parts = 1024 / n_pad;  // 4 .. 32
+  const int groups = (F + 31) / 32;
+  const int per = (groups + parts - 1) / parts;
+  const int p = tid / n_pad, x = tid - p * n_pad;
+  const int g0 = p * per, g1 = min(groups, g0 + per);
+  int sum = 0;
+  if (x < N)
+    for (int g = g0; g < g1; ++g) sum += gcnt[g * N + x];
+  part[tid] = sum;
+  __syncthreads();
+  int total = 0;
+  if (tid < N)
+    for (int q = 0; q < parts; ++q) {  // exclusive over the parts of expert tid
+      const int v = part[q * n_pad + tid];
+      part[q * n_pad + tid] = total;
+      total += v;
     }
-    if (lane < kWarps) sh[lane] = s;
+  int all_rows, all_tiles;
+  const int off = block_exclusive_scan<32>(total, sh, &all_rows);
+  const int tstart = block_exclusive_scan<32>((total + tile_rows - 1) / tile_rows, sh, &all_tiles);
+  if (tid < N) {
+    counts[tid] = total;
+    offsets[tid] = off;
+    ex_off[tid] = off;
+    ex_tile[tid] = tstart;
+  }
+  if (tid == 0) {
+    offsets[N] = all_rows;
+    ex_off[N] = all_rows;
+    ex_tile[N] = all_tiles;
   }
   __syncthreads();
-  const int incl = x + (w > 0 ? sh[w - 1] : 0);
-  *total = sh[kWarps - 1];
+  if (x < N) {
+    int run = ex_off[x] + part[tid];
+    for (int g = g0; g < g1; ++g) {
+      const int c = gcnt[g * N + x];
+      gcnt[g * N + x] = run;
+      run += c;
+    }
+  }
+  write_tile_table(N, T, k, n_shared, tile_rows, ex_off, ex_tile, tiles, num_tiles, ready);
   __syncthreads();
-  return incl - v;
+  if (tid < F) {
+    if (e >= 0) {
+      const int pos = gcnt[w * N + e] + __popc(same & lanemask_lt());
+      perm[pos] = tid;
+      inv[tid] = pos;
+    } else {
+      inv[tid] = -1;
+    }
+  }
 }
 
-// Hist, scan and place in one cooperative launch (N % 4 == 0, N <= 256; grid resident).
-__global__ void __launch_bounds__(kDispatchChunk)
+size_t small_smem_bytes(int N) {
+  return sizeof(int) * (static_cast<size_t>(kSmallGroups) * N + 2 * N + 2);
+}
+
+// Hist, scan and place in one cooperative launch (N % 4 == 0, N <= 256; grid resident): blocks of
+// kThr threads, kSlots slots per thread (f = base + c kThr + tid).  <256, 1> for most batches;
+// <1024, 2> for those whose 256-slot blocks are not resident at once or so many that every block
+// reading the whole histogram costs more (fused_dispatch_shape).
+template <int kThr, int kSlots>
+__global__ void __launch_bounds__(kThr)
     dispatch_fused_kernel(const int32_t* __restrict__ idx, int64_t F, int k, int N, int64_t T,
                           int n_shared, int tile_rows, int32_t* blk_hist, int32_t* __restrict__ counts,
                           int32_t* __restrict__ offsets, int32_t* __restrict__ perm,
                           int32_t* __restrict__ inv, TileEntry* __restrict__ tiles,
                           int32_t* __restrict__ num_tiles, unsigned int* sync_ctr,
                           int32_t* status, int32_t* __restrict__ ready) {
+  constexpr int kGroups = kThr / 32 * kSlots;  // groups of 32 slots
   extern __shared__ int dsm[];
-  int* wcnt = dsm;                   // [kWarps][N] per-warp counts, then per-warp bases
-  int* tot = wcnt + kWarps * N;      // [N] slots of each expert over all blocks
+  int* wcnt = dsm;                   // [kGroups][N] per-group counts, then per-group bases
+  int* tot = wcnt + kGroups * N;      // [N] slots of each expert over all blocks
   int* pre = tot + N;                // [N] slots of each expert in the blocks before this one
   int* ex_off = pre + N;             // [N+1]
   int* ex_tile = ex_off + N + 1;     // [N+1]
@@ -293,23 +363,30 @@ __global__ void __launch_bounds__(kDispatchChunk)
   pdl_trigger();
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int nblk = static_cast<int>(gridDim.x), b = static_cast<int>(blockIdx.x);
-  for (int i = tid; i < kWarps * N; i += blockDim.x) wcnt[i] = 0;
-  for (int i = tid; i < N; i += blockDim.x) {
+  for (int i = tid; i < kGroups * N; i += kThr) wcnt[i] = 0;
+  for (int i = tid; i < N; i += kThr) {
     tot[i] = 0;
     pre[i] = 0;
   }
   __syncthreads();
-  // ---- 1. this block's slots: validity, per-warp counts, block histogram
-  const int64_t f = static_cast<int64_t>(b) * kDispatchChunk + tid;
-  int e = -1;
-  if (f < F && !slot_valid(idx, f, k, N, &e) && status != nullptr)
-    atomicOr(status, PR2_STATUS_BAD_INDEX);
-  const unsigned same = __match_any_sync(0xffffffffu, e);
-  if (e >= 0 && lane == __ffs(same) - 1) wcnt[w * N + e] = __popc(same);
+  // ---- 1. this block's slots: validity, per-group counts, block histogram
+  const int64_t f0 = static_cast<int64_t>(b) * (kThr * kSlots);
+  int e[kSlots];
+  unsigned same[kSlots];
+#pragma unroll
+  for (int c = 0; c < kSlots; ++c) {
+    const int64_t f = f0 + c * kThr + tid;
+    e[c] = -1;
+    if (f < F && !slot_valid(idx, f, k, N, &e[c]) && status != nullptr)
+      atomicOr(status, PR2_STATUS_BAD_INDEX);
+    same[c] = __match_any_sync(0xffffffffu, e[c]);
+    if (e[c] >= 0 && lane == __ffs(same[c]) - 1)
+      wcnt[(c * (kThr / 32) + w) * N + e[c]] = __popc(same[c]);
+  }
   __syncthreads();
-  for (int x = tid; x < N; x += blockDim.x) {
+  for (int x = tid; x < N; x += kThr) {
     int c = 0;
-    for (int ww = 0; ww < kWarps; ++ww) c += wcnt[ww * N + x];
+    for (int ww = 0; ww < kGroups; ++ww) c += wcnt[ww * N + x];
     blk_hist[static_cast<int64_t>(b) * N + x] = c;
   }
   // ---- grid barrier (every block is resident: cooperative launch); bounded
@@ -332,7 +409,7 @@ __global__ void __launch_bounds__(kDispatchChunk)
   __syncthreads();
   if (abort_s) return;
   // ---- 2. expert totals and this block's prefix from the whole histogram (int4 columns)
-  const int n4 = N / 4, G = kDispatchChunk / n4;
+  const int n4 = N / 4, G = kThr / n4;
   const int q = tid % n4, g = tid / n4;
   if (g < G) {
     int4 all = make_int4(0, 0, 0, 0), before = make_int4(0, 0, 0, 0);
@@ -371,10 +448,9 @@ __global__ void __launch_bounds__(kDispatchChunk)
   __syncthreads();
   int all_rows, all_tiles;
   const int total = tid < N ? tot[tid] : 0;
-  const int off = block256_exclusive_scan(total, sh, &all_rows);
-  const int tstart =
-      block256_exclusive_scan(tid < N ? (total + tile_rows - 1) / tile_rows : 0, sh,
-                              &all_tiles);
+  const int off = block_exclusive_scan<kThr / 32>(total, sh, &all_rows);
+  const int tstart = block_exclusive_scan<kThr / 32>(
+      tid < N ? (total + tile_rows - 1) / tile_rows : 0, sh, &all_tiles);
   if (tid < N) {
     ex_off[tid] = off;
     ex_tile[tid] = tstart;
@@ -392,19 +468,23 @@ __global__ void __launch_bounds__(kDispatchChunk)
     if (tid == 0) offsets[N] = all_rows;
     write_tile_table(N, T, k, n_shared, tile_rows, ex_off, ex_tile, tiles, num_tiles, ready);
   }
-  // ---- 3. stable placement: per-warp bases, then ranks within the warp
-  for (int x = tid; x < N; x += blockDim.x) {
+  // ---- 3. stable placement: per-group bases, then ranks within the group
+  for (int x = tid; x < N; x += kThr) {
     int run = ex_off[x] + pre[x];
-    for (int ww = 0; ww < kWarps; ++ww) {
+    for (int ww = 0; ww < kGroups; ++ww) {
       const int c = wcnt[ww * N + x];
       wcnt[ww * N + x] = run;
       run += c;
     }
   }
   __syncthreads();
-  if (f < F) {
-    if (e >= 0) {
-      const int pos = wcnt[w * N + e] + __popc(same & lanemask_lt());
+#pragma unroll
+  for (int c = 0; c < kSlots; ++c) {
+    const int64_t f = f0 + c * kThr + tid;
+    if (f >= F) continue;
+    if (e[c] >= 0) {
+      const int pos =
+          wcnt[(c * (kThr / 32) + w) * N + e[c]] + __popc(same[c] & lanemask_lt());
       perm[pos] = static_cast<int32_t>(f);
       inv[f] = pos;
     } else {
@@ -494,9 +574,9 @@ __global__ void __launch_bounds__(kHistBlock)
   __syncthreads();
   int all_rows, all_tiles;
   const int total = tid < N ? tot[tid] : 0;
-  const int off = block_exclusive_scan(total, sh, &all_rows);
+  const int off = block_exclusive_scan<32>(total, sh, &all_rows);
   const int tstart =
-      block_exclusive_scan(tid < N ? (total + tile_rows - 1) / tile_rows : 0, sh, &all_tiles);
+      block_exclusive_scan<32>(tid < N ? (total + tile_rows - 1) / tile_rows : 0, sh, &all_tiles);
   if (tid < N) {
     ex_off[tid] = off;
     ex_tile[tid] = tstart;
@@ -531,36 +611,61 @@ __global__ void __launch_bounds__(kHistBlock)
   }
 }
 
+constexpr int kFewBlocks = 384;
+
 size_t hist_smem_bytes(int N) { return sizeof(int) * (static_cast<size_t>(kHistWarps) * N + 4 * N + 2); }
 
-size_t fused_smem_bytes(int N) { return sizeof(int) * (static_cast<size_t>(kWarps) * N + 4 * N + 2); }
+size_t fused_smem_bytes(int N, int groups) {
+  return sizeof(int) * (static_cast<size_t>(groups) * N + 4 * N + 2);
+}
 
-// Whether the fused dispatch can run (shape, and every block resident at once), cached per
-// device and N.
-bool fused_dispatch_ok(int N, int nblk, int num_sms) {
-  if (N % 4 != 0 || N > kDispatchChunk || nblk < 1) return false;
+cudaError_t set_large_fused_smem(int N) {
+  return cudaFuncSetAttribute(dispatch_fused_kernel<1024, 2>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(fused_smem_bytes(N, 64)));
+}
+
+// Blocks of the fused dispatch that fit on one SM (0 on error), cached per device, N and shape.
+int fused_blocks_per_sm(int N, bool large) {
   struct Entry {
-    int dev, N, blocks_per_sm;
+    int dev, N, large, blocks_per_sm;
   };
   static std::mutex mu;
-  static Entry cache[32];
+  static Entry cache[64];
   static int used = 0;
   int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   std::lock_guard<std::mutex> lock(mu);
-  int per_sm = -1;
   for (int i = 0; i < used; ++i)
-    if (cache[i].dev == dev && cache[i].N == N) per_sm = cache[i].blocks_per_sm;
-  if (per_sm < 0) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, dispatch_fused_kernel,
-                                                      kDispatchChunk, fused_smem_bytes(N)) !=
-        cudaSuccess) {
-      (void)cudaGetLastError();
-      per_sm = 0;
-    }
-    if (used < 32) cache[used++] = Entry{dev, N, per_sm};
+    if (cache[i].dev == dev && cache[i].N == N && cache[i].large == static_cast<int>(large))
+      return cache[i].blocks_per_sm;
+  int per_sm = 0;
+  const cudaError_t err =
+      large ? set_large_fused_smem(N) : cudaSuccess;
+  if (err != cudaSuccess ||
+      (large ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                   &per_sm, dispatch_fused_kernel<1024, 2>, 1024, fused_smem_bytes(N, 64))
+             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                   &per_sm, dispatch_fused_kernel<kDispatchChunk, 1>, kDispatchChunk,
+                   fused_smem_bytes(N, kWarps))) != cudaSuccess) {
+    (void)cudaGetLastError();
+    per_sm = 0;
   }
-  return static_cast<int64_t>(per_sm) * num_sms >= nblk;
+  if (used < 64) cache[used++] = Entry{dev, N, static_cast<int>(large), per_sm};
+  return per_sm;
+}
+
+// Shape of the fused dispatch for F slots: 1 = 256-slot blocks, 2 = 2048-slot blocks, 0 = cannot
+// run (every block has to be resident).  Every block reads the whole histogram, which past ~400
+// blocks of 256 slots costs more than blocks of 2048 slots lose in parallelism (N = 128, k = 8,
+// stage times: T = 8192 17.0 us small, T = 16384 22.7 small / 19.5 large; T = 32768, where the small
+// blocks are not resident at once, 37.8 us as three kernels / 19.5 large; N = 256 57 / 21).
+int fused_dispatch_shape(int N, int64_t F, int num_sms) {
+  if (N % 4 != 0 || N > kDispatchChunk || F < 1) return 0;
+  const int64_t small = (F + kDispatchChunk - 1) / kDispatchChunk, large = (F + 2047) / 2048;
+  if (small <= kFewBlocks && small <= static_cast<int64_t>(fused_blocks_per_sm(N, false)) * num_sms)
+    return 1;
+  return large <= static_cast<int64_t>(fused_blocks_per_sm(N, true)) * num_sms ? 2 : 0;
 }
 
 template <typename T, int V, int KMAX>  // V elements per 16-byte vector, k <= KMAX
@@ -812,20 +917,34 @@ cudaError_t launch_dispatch(const DispatchArgs& a, int num_sms, cudaStream_t st)
   const int64_t F = a.T * a.k;
   const int nblk = static_cast<int>((F + kDispatchChunk - 1) / kDispatchChunk);
   cudaError_t err = cudaSuccess;
-  if (nblk > 0 && a.sync_ctr != nullptr && fused_dispatch_ok(a.N, nblk, num_sms)) {
+  // One block for a small batch, any N (stage times with N = 128, k = 8: 128 slots 10.8 us by the
+  // cooperative launch, 10.1 in one block; 512 11.9 / 10.5; 2048, two slots per thread 13.2 / 13.7)
+  if (F > 0 && F <= kSmallSlots) {
+    const size_t smem = small_smem_bytes(a.N);
+    err = cudaFuncSetAttribute(dispatch_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               static_cast<int>(smem));
+    if (err != cudaSuccess) return err;
+    return launch_pdl(dispatch_small_kernel, dim3(1), dim3(1024), smem, st, 1, a.idx,
+                      static_cast<int>(F), a.k, a.N, a.T, a.n_shared, a.tile_rows, a.counts,
+                      a.offsets, a.perm, a.inv, a.tiles, a.num_tiles, a.status, a.ready);
+  }
+  const int shape = a.sync_ctr != nullptr ? fused_dispatch_shape(a.N, F, num_sms) : 0;
+  if (shape != 0) {
     err = cudaMemsetAsync(a.sync_ctr, 0, sizeof(unsigned int), st);
+    if (err == cudaSuccess && shape == 2) err = set_large_fused_smem(a.N);
     if (err != cudaSuccess) return err;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nblk);
-    cfg.blockDim = dim3(kDispatchChunk);
-    cfg.dynamicSmemBytes = fused_smem_bytes(a.N);
+    cfg.gridDim = dim3(shape == 2 ? static_cast<unsigned>((F + 2047) / 2048) : nblk);
+    cfg.blockDim = dim3(shape == 2 ? 1024 : kDispatchChunk);
+    cfg.dynamicSmemBytes = fused_smem_bytes(a.N, shape == 2 ? 64 : kWarps);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;  // blocks wait on one another once
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    err = cudaLaunchKernelEx(&cfg, dispatch_fused_kernel, a.idx, F, a.k, a.N, a.T, a.n_shared,
+    auto* kern = shape == 2 ? dispatch_fused_kernel<1024, 2> : dispatch_fused_kernel<kDispatchChunk, 1>;
+    err = cudaLaunchKernelEx(&cfg, kern, a.idx, F, a.k, a.N, a.T, a.n_shared,
                              a.tile_rows, a.blk_hist, a.counts, a.offsets, a.perm, a.inv, a.tiles,
                              a.num_tiles, a.sync_ctr, a.status, a.ready);
     if (err != cudaSuccess) return err;

@@ -52,11 +52,13 @@ __global__ void __launch_bounds__((SimtTile<BM, BN, TM, TN, BK, kSwiglu>::kThrea
   constexpr int kSub = kMinTileRows / BM;  // row blocks of one M-tile
   pdl_wait();
   pdl_trigger();
-  // mt < max_tiles by the grid; a dispatch that timed out leaves the table unwritten
+  // mt < max_tiles by the grid; a dispatch that timed out leaves the table unwritten.  The three
+  // loads are in flight together.
   const int row_block = static_cast<int>(blockIdx.x) / col_blocks;
   const int mt = row_block / kSub;
-  if (status_timed_out(g.status) || mt >= *g.num_tiles) return;
+  const int nm = *g.num_tiles;
   const TileEntry te = g.tiles[mt];
+  if (status_timed_out(g.status) || mt >= nm) return;
   const int K = g.K, n_out = g.n_out;
   const float* __restrict__ A = g.A;
   const bool shared = te.expert >= g.N;

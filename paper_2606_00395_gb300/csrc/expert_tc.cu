@@ -309,8 +309,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ int jobs_ready;  // jobs [0, jobs_ready) of this CTA may read their rows
   if (threadIdx.x == 0) {
     jobs_ready = 0;
-    const int nm = status_timed_out(ma.status) ? 0 : *ma.num_tiles;
-    nm_s = nm < 0 ? 0 : (nm > ma.max_tiles ? ma.max_tiles : nm);
+    const int nm = *ma.num_tiles;  // in flight with the status word
+    nm_s = status_timed_out(ma.status) || nm < 0 ? 0 : (nm > ma.max_tiles ? ma.max_tiles : nm);
   }
   __syncthreads();
   Schedule sch;  // dispatch's tile count, never above the host bound; 0 after a timeout
