@@ -44,8 +44,10 @@
 // (up), one column per row of the tile.  Columns fall into two row halves, 0 = rows 0-127 and
 // 1 = rows 128-255, each with its own full / empty barriers.  A job of at most 128 rows uses one
 // of them, alternating, so that its epilogue overlaps the next job's MMAs.  A larger job uses
-// both; its last kSplit K blocks are multiplied for row half 0 first, and its first ones likewise
-// if half 1 is still being drained, so that the epilogue of one half overlaps MMAs of the other.
+// both; its last K block is multiplied for row half 0 first, and its first one likewise if half 1
+// is still being drained, so that the epilogue of one half overlaps MMAs of the other (three such K
+// blocks overlap more, but MMAs of N = 128 take more shared-memory reads per FLOP: T = 3001 replay
+// 272.5 us with three, 265.9 with one, 271.2 with none).
 #include "pr2_device.cuh"
 #include "pr2_internal.h"
 
@@ -79,7 +81,6 @@ struct Ring {
   static constexpr int kOut = kRRing + kStagesR * kRStage;      // epilogue buffers
   static constexpr int kBarOffset = kOut + 4 * kOutBuf;  // two per side
   static constexpr int kSmemBytes = 1024 + kBarOffset + 256;
-  static constexpr int kSplit = kStagesR;  // K blocks multiplied one row half at a time
   static_assert(kStagesW / 2 + 1 < kRel && kStagesR < kRel, "a ring could see a release twice");
   static_assert((2 * kRel + 5) * 8 + 8 <= 256, "barrier area");
 };
@@ -455,52 +456,30 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         if (ok) commit(&acc_full[h]);
       } else {
-        constexpr int kSplit = R::kSplit;
         constexpr uint32_t idesc0 = umma_idesc_bf16(128, kHalfRows);
         const uint32_t idesc1 = umma_idesc_bf16(128, n - kHalfRows);
-        Stage hs[kSplit];
         ok = wait_empty(0);
         int kb = 0;
         const uint32_t par1 = ((par_empty >> 1) & 1u) ^ 1u;
         const bool free1 = __all_sync(0xffffffffu, mbar_test_wait(&acc_empty[1], par1));
-        if (ok && KB > 2 * kSplit && !free1) {
-          // half 1 is still being drained: the first K blocks' half 0 goes ahead
-#pragma unroll
-          for (int j = 0; j < kSplit; ++j) {
-            if (ok) ok = acquire(hs[j]);
-            if (ok) multiply(hs[j], 0, idesc0, 0, j == 0, nullptr);
-          }
+        if (ok && KB > 1 && !free1) {
+          // half 1 is still being drained: the first K block's half 0 goes ahead
+          ok = acquire(st);
+          if (ok) multiply(st, 0, idesc0, 0, true, nullptr);
           if (ok) ok = wait_empty(1);
-          if (ok) {
-#pragma unroll
-            for (int j = 0; j < kSplit; ++j)
-              multiply(hs[j], kHalfRows, idesc1, kHalfRows, j == 0, next_rel());
-          }
-          kb = kSplit;
+          if (ok) multiply(st, kHalfRows, idesc1, kHalfRows, true, next_rel());
+          kb = 1;
         } else if (ok) {
           ok = wait_empty(1);
         }
         if (ok) ok = acquire(st);
-        const int tail = KB - kb < kSplit ? KB - kb : kSplit;  // K blocks of the split end
-        for (; kb < KB - tail && ok; ++kb) {
+        for (; kb < KB - 1 && ok; ++kb) {
           multiply(st, 0, idesc, 0, kb == 0, next_rel());
           ok = acquire(st);
         }
-        hs[0] = st;
-#pragma unroll
-        for (int j = 0; j < kSplit; ++j) {
-          if (j < tail && ok) {
-            if (j > 0) ok = acquire(hs[j]);
-            if (ok)
-              multiply(hs[j], 0, idesc0, 0, kb + j == 0,
-                       j == tail - 1 ? &acc_full[0] : nullptr);
-          }
-        }
         if (ok) {
-#pragma unroll
-          for (int j = 0; j < kSplit; ++j)
-            if (j < tail)
-              multiply(hs[j], kHalfRows, idesc1, kHalfRows, kb + j == 0, next_rel());
+          multiply(st, 0, idesc0, 0, kb == 0, &acc_full[0]);
+          multiply(st, kHalfRows, idesc1, kHalfRows, kb == 0, next_rel());
           commit(&acc_full[1]);
         }
       }
