@@ -15,17 +15,21 @@
 // (S = 1), each CTA takes half the pipeline stages so that two run on an SM side by side, one
 // CTA's loads and finishing overlapping the other's MMAs (RouteTcArgs::compact).
 //
-// Warp roles: warp 0 = TMA producer, warp 1 = TMEM owner and MMA issuer, warps 2..5 = epilogue.
+// Warp roles: warp 0 = TMA producer, warp 1 = TMEM owner and MMA issuer, warps 2..5 = epilogue
+// (by warps, below: all sixteen).
 // With S > 1 the partials are reduce-scattered by rows through distributed shared memory: CTA q
 // receives rows [q 128/S, (q+1) 128/S) of every CTA's partial, stored [source][column/4][row][4]
 // so that each warp store moves contiguous bytes; rows beyond the batch are not moved.  Two ways
 // to finish the rows:
-//  - by warps (predict with 64 < N <= 128, S >= 4): all six warps sum the S copies once, in source
-//    order (deterministic), into rows of shared memory, and each then finishes whole rows, up to
-//    six at a time: a lane holds four experts, and the top k + 1 come out one by one by warp maxima
-//    (redux.sync) over orderable 32-bit values.  Sum and rows of a T = 256 predict call: 4.4 us by
-//    threads, 2.9 us by warps (3.7 with five shuffles instead of redux.sync); eight experts per
-//    lane (N = 256, 64 rows per CTA) 24 us where threads take 11.
+//  - by warps (N <= 128, S >= 4; CTAs of sixteen warps): the warps sum the S copies once, in source
+//    order (deterministic), into rows of shared memory, and each then finishes kRows whole rows, a
+//    lane holding four experts.  predict: the top k + 1 come out one by one by warp maxima
+//    (redux.sync) over orderable 32-bit values.  loss: the dKL/dz rows leave transposed through
+//    shared memory.  Short chains of ALU work per element bound this, not the shuffles or
+//    reductions, so it is the number of warps that counts: calls by threads / six warps / sixteen,
+//    N = 128: predict T = 4001 16.5 / 16.2 / 13.9 us, T = 600 12.9 / 11.1 / 10.3; loss T_c = 2048
+//    18.9 / 21.1 / 17.9; by threads / sixteen warps replay T = 4001 12.4 / 10.4, T = 256 8.9 / 7.5;
+//    predict with N = 64, T = 4096 11.1 / 9.6.
 //  - by threads (everything else): the four epilogue warps sum the S copies in place, walking
 //    consecutive 16-byte words so that no two lanes of a warp hit one bank.  Each row is then
 //    finished by S consecutive threads, thread `part` owning experts [part N/S, (part+1) N/S);
@@ -47,6 +51,7 @@ namespace pr2 {
 namespace {
 
 constexpr int kThreads = 192;
+constexpr int kWarpThreads = 512;                // CTAs whose rows are finished by warps
 constexpr int kBK = 64;                          // bf16 elements per 128-byte swizzle row
 constexpr int kATileBytes = kTileM * kBK * 2;    // 16 KB
 constexpr int kKeep = kMaxTopK + 1;              // top-(k+1) kept for the margin
@@ -87,19 +92,14 @@ __host__ __device__ inline RouteSmemLayout route_layout(int N, bool predict, boo
 // stages once every CTA of the cluster has finished its K blocks.
 __host__ __device__ inline int route_recv_bytes(int b_rows) { return b_rows * kTileM * 4; }
 
-// Whether predict rows are finished by warps: 16 or 32 rows per CTA of more than 64 experts (calls
-// with N = 128: T = 600, S = 8 13.0 us by threads, 11.1 by warps; T = 4001, S = 4 16.4 / 16.15;
-// T = 8192, S = 2 21.8 / 25.2; N = 64, T = 4096, S = 4 11.1 / 11.7).
+// Whether rows are finished by warps.
 __host__ __device__ inline bool route_by_warps(int N, int split) {
-  return N > 64 && N <= 128 && split >= 4;
+  return N <= 128 && split >= 4;
 }
-// The rows that they move into row order at a time, behind the received copies: the largest power
-// of two (at most the CTA's rows) that fits.
-__host__ __device__ inline int route_finish_rows(const RouteSmemLayout& L, int split) {
-  const int row = (L.b_rows / 4 + 1) * 16;
-  int rc = 1;
-  while (rc < kTileM / split && route_recv_bytes(L.b_rows) + 2 * rc * row <= L.bar_offset) rc *= 2;
-  return rc;
+// Shared memory that this takes: the received copies, the rows in row order and (loss) bf16 rows.
+__host__ __device__ inline int route_warps_bytes(const RouteSmemLayout& L, int split) {
+  const int rows = kTileM / split;
+  return route_recv_bytes(L.b_rows) + rows * ((L.b_rows / 4 + 1) * 16 + L.b_rows * 2 + 8);
 }
 
 __host__ __device__ inline uint32_t tmem_cols_for(int cols) {
@@ -201,10 +201,23 @@ __device__ __forceinline__ uint32_t order_bits(float z) {
 __device__ __forceinline__ float order_value(uint32_t ord) {
   return __uint_as_float((ord & 0x80000000u) ? (ord & 0x7fffffffu) : ~ord);
 }
-__device__ __forceinline__ float warp_add(float v) {
+// Warp-wide operations on kRB rows at once: a warp issues in order, so each step is written for all
+// rows before the next one.
+template <int kRB>
+__device__ __forceinline__ void warp_add(float (&v)[kRB]) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+  for (int o = 16; o > 0; o >>= 1) {
+    float w[kRB];
+#pragma unroll
+    for (int j = 0; j < kRB; ++j) w[j] = __shfl_xor_sync(0xffffffffu, v[j], o);
+#pragma unroll
+    for (int j = 0; j < kRB; ++j) v[j] += w[j];
+  }
+}
+template <int kRB>
+__device__ __forceinline__ void warp_max(uint32_t (&v)[kRB]) {
+#pragma unroll
+  for (int j = 0; j < kRB; ++j) v[j] = __reduce_max_sync(0xffffffffu, v[j]);
 }
 
 // Finishes kRB predict rows by one warp (N <= 128).  Row j: [p_old | b] of 2 N floats at rows[j] in
@@ -223,7 +236,8 @@ __device__ __forceinline__ int finish_predict_rows(const float4* const (&rows)[k
   const int n4 = a.N / 4;
   uint32_t key[kRB][4];
   uint32_t ids[kRB];  // the lane's experts in the order of its keys, 4 bits each
-  float mx[kRB], sum[kRB], my_z[kRB];
+  uint32_t head[kRB];
+  float mx[kRB], sum[kRB], my_z[kRB], zs[kRB][4];
   int my_e[kRB];
 #pragma unroll
   for (int j = 0; j < kRB; ++j) {
@@ -259,27 +273,43 @@ __device__ __forceinline__ int finish_predict_rows(const float4* const (&rows)[k
         id[q + 1] = sw ? i0 : id[q + 1];
       }
     ids[j] = id[0] | id[1] << 4 | id[2] << 8 | id[3] << 12;
-    mx[j] = fmaxf(order_value(__reduce_max_sync(0xffffffffu, key[j][0])), -FLT_MAX);
-    sum[j] = 0.f;
-    if (lane < n4)
+    head[j] = key[j][0];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) sum[j] += expf(z[q] - mx[j]);
+    for (int q = 0; q < 4; ++q) zs[j][q] = z[q];
     my_z[j] = 0.f;
     my_e[j] = 0;
   }
+  warp_max<kRB>(head);
+#pragma unroll
+  for (int j = 0; j < kRB; ++j) {
+    mx[j] = fmaxf(order_value(head[j]), -FLT_MAX);
+    sum[j] = 0.f;
+    if (lane < n4)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) sum[j] += expf(zs[j][q] - mx[j]);
+  }
+  warp_add<kRB>(sum);
   const int rounds = a.k < a.N ? a.k + 1 : a.k;
   for (int r = 0; r < rounds; ++r) {
+    unsigned has[kRB];
+    int e[kRB];
+    if (r > 0) {
+#pragma unroll
+      for (int j = 0; j < kRB; ++j) head[j] = key[j][0];
+      warp_max<kRB>(head);
+    }
+#pragma unroll
+    for (int j = 0; j < kRB; ++j) has[j] = __ballot_sync(0xffffffffu, key[j][0] == head[j]);
+#pragma unroll
+    for (int j = 0; j < kRB; ++j)
+      e[j] = __shfl_sync(0xffffffffu, lane * 4 + static_cast<int>(ids[j] & 15u), __ffs(has[j]) - 1);
 #pragma unroll
     for (int j = 0; j < kRB; ++j) {
-      const uint32_t m = __reduce_max_sync(0xffffffffu, key[j][0]);
-      const unsigned has = __ballot_sync(0xffffffffu, key[j][0] == m);
-      const int owner = __ffs(has) - 1;
-      const int e = __shfl_sync(0xffffffffu, lane * 4 + static_cast<int>(ids[j] & 15u), owner);
       if (lane == r) {
-        my_z[j] = order_value(m);
-        my_e[j] = e;
+        my_z[j] = order_value(head[j]);
+        my_e[j] = e[j];
       }
-      if (lane == owner) {
+      if (lane == e[j] >> 2) {
 #pragma unroll
         for (int q = 0; q < 3; ++q) key[j][q] = key[j][q + 1];
         key[j][3] = 0u;
@@ -287,25 +317,145 @@ __device__ __forceinline__ int finish_predict_rows(const float4* const (&rows)[k
       }
     }
   }
+  float pr[kRB], sk[kRB], pk[kRB], pk1[kRB];
+#pragma unroll
+  for (int j = 0; j < kRB; ++j) {
+    pr[j] = expf(my_z[j] - mx[j]) * (1.0f / sum[j]);
+    sk[j] = lane < a.k ? pr[j] : 0.f;
+  }
+  if (a.norm) warp_add<kRB>(sk);
+#pragma unroll
+  for (int j = 0; j < kRB; ++j) pk[j] = __shfl_sync(0xffffffffu, pr[j], a.k - 1);
+#pragma unroll
+  for (int j = 0; j < kRB; ++j) pk1[j] = __shfl_sync(0xffffffffu, pr[j], a.k);  // k <= 8
   int ties = 0;
 #pragma unroll
   for (int j = 0; j < kRB; ++j) {
-    const float pr = expf(my_z[j] - mx[j]) * (1.0f / warp_add(sum[j]));
-    const float sk = a.norm ? warp_add(lane < a.k ? pr : 0.f) : 0.f;
     if (live[j] && lane < a.k) {
       a.idx_out[t[j] * a.k + lane] = my_e[j];
-      a.gates[t[j] * a.k + lane] = a.norm ? pr * (1.0f / sk) : pr;
+      a.gates[t[j] * a.k + lane] = a.norm ? pr[j] * (1.0f / sk[j]) : pr[j];
       if (count) atomicAdd(&hist[my_e[j]], 1);
     }
-    const float pk = __shfl_sync(0xffffffffu, pr, a.k - 1);
-    const float pk1 = __shfl_sync(0xffffffffu, pr, a.k);  // k <= 8
-    ties += (live[j] && a.k < a.N && pk - pk1 < (float)PR2_NEAR_TIE_GAP) ? 1 : 0;
+    ties += (live[j] && a.k < a.N && pk[j] - pk1[j] < (float)PR2_NEAR_TIE_GAP) ? 1 : 0;
   }
   return ties;
 }
 
-template <int kMode, int split>
-__global__ void __launch_bounds__(kThreads, 1)
+// kRB replay rows finished by one warp: row j's logits are N floats at rows[j] (lane l: experts
+// 4 l ..), lane s < k holds cached slot s in es[j] (-1: none, out of range or repeated).  Writes
+// the gates (divided by their sum over the valid slots under PR2_F_NORMALIZE_TOPK) and, where
+// asked for, the row of rho.
+template <int kRB>
+__device__ __forceinline__ void finish_replay_rows(const float4* const (&rows)[kRB],
+                                                   const int (&es)[kRB], const int64_t (&t)[kRB],
+                                                   const bool (&live)[kRB], const RouteTcArgs& a) {
+  const int lane = threadIdx.x & 31;
+  const int n4 = a.N / 4;
+  float4 z[kRB];
+  uint32_t head[kRB];
+  float sum[kRB], g[kRB], sk[kRB];
+#pragma unroll
+  for (int j = 0; j < kRB; ++j) {
+    z[j] = lane < n4 ? rows[j][lane] : make_float4(-FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX);
+    head[j] = order_bits(fmaxf(fmaxf(z[j].x, z[j].y), fmaxf(z[j].z, z[j].w)));
+  }
+  warp_max<kRB>(head);
+#pragma unroll
+  for (int j = 0; j < kRB; ++j) {
+    const float mx = fmaxf(order_value(head[j]), -FLT_MAX);
+    const float zg = es[j] >= 0 ? reinterpret_cast<const float*>(rows[j])[es[j]] : 0.f;
+    z[j].x = expf(z[j].x - mx);
+    z[j].y = expf(z[j].y - mx);
+    z[j].z = expf(z[j].z - mx);
+    z[j].w = expf(z[j].w - mx);
+    sum[j] = lane < n4 ? (z[j].x + z[j].y) + (z[j].z + z[j].w) : 0.f;
+    g[j] = es[j] >= 0 ? expf(zg - mx) : 0.f;
+  }
+  warp_add<kRB>(sum);
+#pragma unroll
+  for (int j = 0; j < kRB; ++j) sk[j] = g[j] = g[j] * (1.0f / sum[j]);
+  if (a.norm) warp_add<kRB>(sk);
+#pragma unroll
+  for (int j = 0; j < kRB; ++j) {
+    if (!live[j]) continue;
+    if (lane < a.k) a.gates[t[j] * a.k + lane] = a.norm && sk[j] > 0.f ? g[j] * (1.0f / sk[j]) : g[j];
+    if (a.logits_or_probs != nullptr && lane < n4) {
+      const float inv = 1.0f / sum[j];
+      reinterpret_cast<float4*>(a.logits_or_probs + t[j] * a.N)[lane] =
+          make_float4(z[j].x * inv, z[j].y * inv, z[j].z * inv, z[j].w * inv);
+    }
+  }
+}
+
+// The loss mode's rows finished by one warp, kRB at a time: row j's predictor logits b are N floats
+// at rows[j] (lane l: experts 4 l ..), its p_old and teacher values po[j], tr[j].  Writes the
+// per-token KL and the bf16 dKL/dz row to gs[j] (shared memory); formulas at the thread-wise form
+// in the kernel.
+template <int kRB>
+__device__ __forceinline__ void finish_loss_rows(const float4* const (&rows)[kRB],
+                                                 const float4 (&po4)[kRB], const float4 (&tr4)[kRB],
+                                                 const bool (&use)[kRB], const int64_t (&t)[kRB],
+                                                 uint2* const (&gs)[kRB], const RouteTcArgs& a) {
+  const int lane = threadIdx.x & 31;
+  const bool delta = a.delta != 0, in = lane < a.N / 4;
+  float v[kRB][4], lt[kRB][4], tg[kRB][4], s1[kRB], s2[kRB], kl[kRB];
+  uint32_t m1[kRB], m2[kRB];  // row maxima (order_bits: no NaN among the candidates)
+#pragma unroll
+  for (int j = 0; j < kRB; ++j) {
+    const float4 b4 = in ? rows[j][lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float b[4] = {b4.x, b4.y, b4.z, b4.w};
+    const float po[4] = {po4[j].x, po4[j].y, po4[j].z, po4[j].w};
+    const float tr[4] = {tr4[j].x, tr4[j].y, tr4[j].z, tr4[j].w};
+    float c1 = -FLT_MAX, c2 = -FLT_MAX;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const bool ok = in && use[j];
+      v[j][q] = ok ? (delta ? b[q] : po[q] + b[q]) : -INFINITY;
+      tg[j][q] = ok ? tr[q] : 0.f;
+      lt[j][q] = ok && tr[q] > 0.f ? __logf(tr[q]) - (delta ? po[q] : 0.f) : -INFINITY;
+      c1 = fmaxf(c1, v[j][q]);
+      c2 = fmaxf(c2, lt[j][q]);
+    }
+    m1[j] = order_bits(c1);
+    m2[j] = order_bits(c2);
+  }
+  warp_max<kRB>(m1);
+  if (delta) warp_max<kRB>(m2);
+#pragma unroll
+  for (int j = 0; j < kRB; ++j) {
+    s1[j] = s2[j] = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      s1[j] += __expf(v[j][q] - order_value(m1[j]));
+      if (delta) s2[j] += __expf(lt[j][q] - order_value(m2[j]));
+    }
+  }
+  warp_add<kRB>(s1);
+  if (delta) warp_add<kRB>(s2);
+#pragma unroll
+  for (int j = 0; j < kRB; ++j) {
+    const float l1 = order_value(m1[j]) + __logf(s1[j]);  // log normalisers
+    const float l2 = delta ? order_value(m2[j]) + __logf(s2[j]) : 0.f;
+    float g[4];
+    kl[j] = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float lp = v[j][q] - l1;  // log prediction
+      const float ltq = lt[j][q] - l2;
+      const float tgt = delta ? (tg[j][q] > 0.f ? __expf(ltq) : 0.f) : tg[j][q];
+      if (tgt > 0.f) kl[j] += tgt * (ltq - lp);
+      g[q] = in && use[j] ? __expf(lp) - tgt : 0.f;
+    }
+    if (in) *gs[j] = make_uint2(pack_bf16x2(g[0], g[1]), pack_bf16x2(g[2], g[3]));
+  }
+  warp_add<kRB>(kl);
+#pragma unroll
+  for (int j = 0; j < kRB; ++j)
+    if (lane == 0 && t[j] < a.T) a.kl_tok[t[j]] = use[j] ? kl[j] : 0.f;
+}
+
+template <int kMode, int split, bool by_warps>
+__global__ void __launch_bounds__(by_warps ? kWarpThreads : kThreads, 1)
     route_tc_kernel(const __grid_constant__ CUtensorMap tm_h,
                     const __grid_constant__ CUtensorMap tm_w,
                     const __grid_constant__ CUtensorMap tm_wp, RouteTcArgs a) {
@@ -338,7 +488,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   // row then meet in the CTA that finishes it, through distributed shared memory, and are not
   // summed.  Otherwise the cluster splits K and the S partial rows are summed.
   const bool psplit = predict && L.passes == 2 && split == 2;
-  const bool by_warps = predict && route_by_warps(N, split);
   const int KBper = psplit ? a.d / kBK : (a.d / kBK) / split;
   const int kb0 = psplit ? 0 : rank * KBper, kb1 = kb0 + KBper;
   const int npass = psplit ? 1 : L.passes;  // passes this CTA streams
@@ -460,7 +609,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 
   // ---------------- epilogue ----------------
-  const bool epi = warp >= 2;
+  const bool epi = warp >= 2 && warp < 6;
   // predict: experts of the rows this CTA finishes, for the dispatch that follows
   __shared__ int hist_s[kMaxExperts];
   const bool count = predict && a.hist != nullptr;
@@ -482,7 +631,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // replay: cached indices, validated (range, duplicates) while the K blocks run
   int e_s[kMaxTopK];
   bool bad = false;
-  if (kMode == kModeReplay) {
+  if (kMode == kModeReplay && !by_warps) {
 #pragma unroll
     for (int s = 0; s < kMaxTopK; ++s) {
       int e = -1;
@@ -507,7 +656,56 @@ __global__ void __launch_bounds__(kThreads, 1)
   float po_s[kLossPre], tr_s[kLossPre];
   int64_t lrow = 0;
   bool okp = false;
-  if (loss && live) {
+  // finished by warps: this warp's rows wr0 .. wr0 + kRows - 1 of the CTA's; loss: their p_old and
+  // teacher values (row pos[t] of rho), loaded while the K blocks run
+  constexpr int kRows = by_warps ? kTileM / split / (kWarpThreads / 32) : 1;
+  static_assert(!by_warps || kRows * split * (kWarpThreads / 32) == kTileM, "whole rows per warp");
+  const int wr0 = warp * kRows;
+  const int64_t tw = static_cast<int64_t>(t0) + static_cast<int64_t>(rank) * R + wr0;
+  float4 po_w[kRows], tr_w[kRows];
+  bool use_w[kRows];
+  int es_w[kRows];  // replay: cached slot `lane` of the row, -1 if it does not count
+  if (kMode == kModeReplay && by_warps) {
+    bool wrong = false;
+#pragma unroll
+    for (int j = 0; j < kRows; ++j) {
+      const bool in = tw + j < a.T && lane < k;
+      es_w[j] = in ? a.idx_in[(tw + j) * k + lane] : -1;
+    }
+#pragma unroll
+    for (int j = 0; j < kRows; ++j) {
+      const int e = es_w[j];
+      bool ok = e >= 0 && e < N;
+#pragma unroll
+      for (int s2 = 0; s2 < kMaxTopK - 1; ++s2) {
+        // a repeat counts against its later slot; an entry out of range repeats nothing
+        const int other = __shfl_sync(0xffffffffu, e, s2);
+        if (s2 < lane && other == e) ok = false;
+      }
+      wrong = wrong || (tw + j < a.T && lane < k && !ok);
+      if (!ok) es_w[j] = -1;
+    }
+    if (wrong && a.status != nullptr) atomicOr(a.status, PR2_STATUS_BAD_INDEX);
+  }
+  if (loss && by_warps) {
+    int32_t pw[kRows];
+#pragma unroll
+    for (int j = 0; j < kRows; ++j)
+      pw[j] = tw + j < a.T && a.pos != nullptr ? a.pos[tw + j] : 0;
+#pragma unroll
+    for (int j = 0; j < kRows; ++j) {
+      const int64_t r = a.pos != nullptr ? static_cast<int64_t>(pw[j]) : tw + j;
+      use_w[j] = tw + j < a.T && r >= 0 && r < a.T_rho;
+      if (tw + j < a.T && !use_w[j] && lane == 0 && a.status != nullptr)
+        atomicOr(a.status, PR2_STATUS_BAD_INDEX);
+      po_w[j] = tr_w[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (use_w[j] && lane < N / 4) {
+        po_w[j] = reinterpret_cast<const float4*>(a.p_old + (tw + j) * N)[lane];
+        tr_w[j] = reinterpret_cast<const float4*>(a.rho + r * N)[lane];
+      }
+    }
+  }
+  if (loss && live && !by_warps) {
     lrow = a.pos != nullptr ? static_cast<int64_t>(a.pos[t]) : t;
     okp = lrow >= 0 && lrow < a.T_rho;
     if (okp) {
@@ -531,16 +729,17 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 
   bool have = false;
-  if (epi) {
+  if (epi || by_warps) {
     // tcgen05.ld is warp-collective: the whole warp reads TMEM or none of it does.
     have = __all_sync(0xffffffffu, mbar_wait(acc_full, 0, abort_flag, a.status));
     if (have) tc_fence_after();
   }
   if (split > 1) {
     cluster_sync();  // every CTA has finished its K blocks: the pipeline stages are free
-    if (epi && have) {
+    if ((epi || by_warps) && have) {
       // Reduce-scatter by rows: this TMEM row goes to CTA row / R as its row row % R, into the
       // slot of source `rank` (K split) or into columns [rank N, (rank + 1) N) (pass split).
+      // With sixteen warps the four of a lane quadrant share its columns.
       float4* recv_w = reinterpret_cast<float4*>(smem);
       const uint32_t dst = static_cast<uint32_t>(row / R);
       const int drow = row - static_cast<int>(dst) * R;
@@ -551,7 +750,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       // warp of such rows skips its loads too
       const bool in_batch = static_cast<int64_t>(t0) + row < a.T;
       const int cols = static_cast<int64_t>(t0) + q * 32 < a.T ? acc_cols : 0;
-      for (int c0 = 0; c0 < cols; c0 += 32) {
+      constexpr int kShare = by_warps ? kWarpThreads / 128 : 1;
+      for (int c0 = by_warps ? (warp >> 2) * 32 : 0; c0 < cols; c0 += 32 * kShare) {
         uint32_t r0[16], r1[16];
         tmem_ld16(trow + c0, r0);
         tmem_ld16(trow + c0 + 16, r1);
@@ -609,55 +809,76 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   };
 
-  if (split >= 4 && by_warps) {
-    // every thread of the CTA is past the cluster barrier: all six warps sum and finish
-    const int rc = route_finish_rows(L, split);
+  if constexpr (by_warps) {
+    // every thread of the CTA is past the cluster barrier: all sixteen warps sum the S copies into
+    // row order and finish kRows rows each
     const int pitch4 = nb4 + 1;  // 16-byte words of a row: odd, so 8 rows take 8 bank groups
     float4* rm = reinterpret_cast<float4*>(smem) + nb4 * kTileM;
-    const int64_t tr = static_cast<int64_t>(t0) + static_cast<int64_t>(rank) * R;
-    int ties = 0;
-    for (int rb = 0; rb < R && tr + rb < a.T; rb += rc) {
-      for (int i = threadIdx.x; i < nb4 * rc; i += kThreads) {
-        const int row_i = i % rc, at = i / rc * R + rb + row_i;
-        float4 v = recv[at];
+    constexpr int kR = kTileM / split;
+    for (int i = threadIdx.x; i < nb4 * kR; i += kWarpThreads) {
+      float4 v = recv[i];
 #pragma unroll
-        for (int src = 1; src < split; ++src) {
-          const float4 w = recv[src * nb4 * R + at];
-          v.x += w.x;
-          v.y += w.y;
-          v.z += w.z;
-          v.w += w.w;
-        }
-        rm[row_i * pitch4 + i / rc] = v;
+      for (int src = 1; src < split; ++src) {
+        const float4 w = recv[src * nb4 * kR + i];
+        v.x += w.x;
+        v.y += w.y;
+        v.z += w.z;
+        v.w += w.w;
       }
-      __syncthreads();
-      if (*abort_flag == 0) {
-        // a warp's rows interleave; the six warps take the rows at hand in one round
-        constexpr int kRB = split == 4 ? 6 : 3;
-        for (int r = warp * kRB; r < rc && tr + rb + r < a.T; r += (kThreads / 32) * kRB) {
-          const float4* rows[kRB];
-          int64_t ts[kRB];
-          bool lv[kRB];
+      rm[(i % kR) * pitch4 + i / kR] = v;
+    }
+    __syncthreads();
+    const bool good = *abort_flag == 0;
+    const float4* rows[kRows];
+    int64_t ts[kRows];
+    bool lv[kRows];
 #pragma unroll
-          for (int j = 0; j < kRB; ++j) {
-            lv[j] = r + j < rc && tr + rb + r + j < a.T;
-            rows[j] = rm + (lv[j] ? r + j : r) * pitch4;
-            ts[j] = tr + rb + r + j;
-          }
-          ties += finish_predict_rows<kRB>(rows, ts, lv, a, count, hist_s);
-        }
+    for (int j = 0; j < kRows; ++j) {
+      rows[j] = rm + (wr0 + j) * pitch4;
+      ts[j] = tw + j;
+      lv[j] = good && ts[j] < a.T;
+    }
+    if constexpr (predict) {
+      int ties = 0;
+      if (good && tw < a.T) ties = finish_predict_rows<kRows>(rows, ts, lv, a, count, hist_s);
+      if (lane == 0 && ties != 0 && a.near_tie != nullptr)
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.near_tie),
+                  static_cast<unsigned long long>(ties));
+      if (count) {  // every row of this CTA counted: publish its histogram row (zeros included)
+        __syncthreads();
+        int32_t* hrow = a.hist + static_cast<int64_t>(blockIdx.x) * N;
+        for (int e = threadIdx.x; e < N; e += kWarpThreads) hrow[e] = hist_s[e];
       }
-      if (rb + rc < R) __syncthreads();  // the rows are read before the next ones take their place
-    }
-    if (lane == 0 && ties != 0 && a.near_tie != nullptr)
-      atomicAdd(reinterpret_cast<unsigned long long*>(a.near_tie),
-                static_cast<unsigned long long>(ties));
-    if (count) {  // every row of this CTA counted: publish its histogram row (zeros included)
+    } else if constexpr (kMode == kModeReplay) {
+      if (tw < a.T) finish_replay_rows<kRows>(rows, es_w, ts, lv, a);
+    } else {
+      // the bf16 dKL/dz rows meet in shared memory and leave transposed, 2 kR bytes per expert
+      uint8_t* gsb = reinterpret_cast<uint8_t*>(rm + kR * pitch4);
+      const int gpitch = N * 2 + 8;
+      uint2* gs[kRows];
+#pragma unroll
+      for (int j = 0; j < kRows; ++j) {
+        gs[j] = reinterpret_cast<uint2*>(gsb + (wr0 + j) * gpitch + lane * 8);
+        use_w[j] = use_w[j] && good;
+      }
+      finish_loss_rows<kRows>(rows, po_w, tr_w, use_w, ts, gs, a);
       __syncthreads();
-      int32_t* hrow = a.hist + static_cast<int64_t>(blockIdx.x) * N;
-      for (int e = threadIdx.x; e < N; e += kThreads) hrow[e] = hist_s[e];
+      // thread (e, part): 8 rows of expert e, one 16-byte store
+      constexpr int kParts = kR / 8;
+      for (int i = threadIdx.x; i < N * kParts; i += kWarpThreads) {
+        const int e = i / kParts, r0 = i % kParts * 8;
+        uint32_t w[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const uint8_t* at = gsb + (r0 + 2 * r) * gpitch + e * 2;
+          w[r] = *reinterpret_cast<const uint16_t*>(at) |
+                 static_cast<uint32_t>(*reinterpret_cast<const uint16_t*>(at + gpitch)) << 16;
+        }
+        *reinterpret_cast<uint4*>(a.gt + static_cast<int64_t>(e) * a.Tpad + t0 + rank * kR + r0) =
+            make_uint4(w[0], w[1], w[2], w[3]);
+      }
     }
-    if (epi) tc_fence_before();
+    tc_fence_before();
   }
   // One pass over this thread's experts, 16 at a time: running max m and sum of exp(z - m),
   // (predict) the top-16 keys, (replay) the z of the cached slots.
@@ -790,7 +1011,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     tc_fence_before();
   }
-  if (epi && loss) {
+  if (epi && loss && !by_warps) {
     // Predictive loss (Eq. pr2_loss, Algorithm 3) of cached row t over experts [fe0, fe0+nr):
     //   standard: prediction Softmax(v), v = p_old + b;  target rho (row pos[t] of the teacher)
     //   delta:    prediction Softmax(b);  target Softmax(u), u = log rho - p_old
@@ -949,29 +1170,30 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (a.late_wait) pdl_wait();
 }
 
-template <int kMode, int kSplit>
+template <int kMode, int kSplit, bool kWarps>
 cudaError_t set_smem_attr(int N) {
-  const cudaError_t err = cudaFuncSetAttribute(route_tc_kernel<kMode, kSplit>,
+  const cudaError_t err = cudaFuncSetAttribute(route_tc_kernel<kMode, kSplit, kWarps>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                route_layout(N, kMode == kModePredict, false).total);
   if (err != cudaSuccess) return err;
   // all of the SM's unified L1 / shared storage as shared memory, so that two compact CTAs fit
-  return cudaFuncSetAttribute(route_tc_kernel<kMode, kSplit>,
+  return cudaFuncSetAttribute(route_tc_kernel<kMode, kSplit, kWarps>,
                               cudaFuncAttributePreferredSharedMemoryCarveout,
                               cudaSharedmemCarveoutMaxShared);
 }
 
-template <int kMode, int kSplit>
-cudaError_t launch_split(const CUtensorMap& tm_h, const CUtensorMap& tm_w,
-                         const CUtensorMap& tm_wp, const RouteTcArgs& a, int tiles,
-                         cudaStream_t st, int* max_clusters) {
-  cudaError_t err = set_smem_attr<kMode, kSplit>(a.N);
+template <int kMode, int kSplit, bool kWarps>
+cudaError_t launch_kernel(const CUtensorMap& tm_h, const CUtensorMap& tm_w,
+                          const CUtensorMap& tm_wp, const RouteTcArgs& a, int tiles,
+                          cudaStream_t st, int* max_clusters) {
+  cudaError_t err = set_smem_attr<kMode, kSplit, kWarps>(a.N);
   if (err != cudaSuccess) return err;
   const size_t smem = route_layout(a.N, kMode == kModePredict, a.compact != 0).total;
+  const dim3 block(kWarps ? kWarpThreads : kThreads);
   if (max_clusters != nullptr) {  // occupancy query only
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(tiles * kSplit);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -980,10 +1202,23 @@ cudaError_t launch_split(const CUtensorMap& tm_h, const CUtensorMap& tm_w,
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaOccupancyMaxActiveClusters(max_clusters, route_tc_kernel<kMode, kSplit>, &cfg);
+    return cudaOccupancyMaxActiveClusters(max_clusters, route_tc_kernel<kMode, kSplit, kWarps>,
+                                          &cfg);
   }
-  return launch_pdl(route_tc_kernel<kMode, kSplit>, dim3(tiles * kSplit), dim3(kThreads), smem,
-                    st, kSplit, tm_h, tm_w, tm_wp, a);
+  return launch_pdl(route_tc_kernel<kMode, kSplit, kWarps>, dim3(tiles * kSplit), block, smem, st,
+                    kSplit, tm_h, tm_w, tm_wp, a);
+}
+
+template <int kMode, int kSplit>
+cudaError_t launch_split(const CUtensorMap& tm_h, const CUtensorMap& tm_w,
+                         const CUtensorMap& tm_wp, const RouteTcArgs& a, int tiles,
+                         cudaStream_t st, int* max_clusters) {
+  if constexpr (kSplit >= 4) {
+    const RouteSmemLayout L = route_layout(a.N, kMode == kModePredict, false);
+    if (route_by_warps(a.N, kSplit) && route_warps_bytes(L, kSplit) <= L.bar_offset)
+      return launch_kernel<kMode, kSplit, true>(tm_h, tm_w, tm_wp, a, tiles, st, max_clusters);
+  }
+  return launch_kernel<kMode, kSplit, false>(tm_h, tm_w, tm_wp, a, tiles, st, max_clusters);
 }
 
 template <int kMode>
@@ -1019,9 +1254,9 @@ cudaError_t launch_any(int mode, const CUtensorMap& tm_h, const CUtensorMap& tm_
 // one SM side by side (a per-CTA %smid / %globaltimer record of a T = 32768 launch).
 template <int kMode>
 int compact_blocks_per_sm(int N) {
-  if (set_smem_attr<kMode, 1>(N) != cudaSuccess) return 0;
+  if (set_smem_attr<kMode, 1, false>(N) != cudaSuccess) return 0;
   cudaFuncAttributes fa{};
-  if (cudaFuncGetAttributes(&fa, route_tc_kernel<kMode, 1>) != cudaSuccess) return 0;
+  if (cudaFuncGetAttributes(&fa, route_tc_kernel<kMode, 1, false>) != cudaSuccess) return 0;
   int dev = 0, smem_sm = 0, reserved = 0, regs_sm = 0, threads_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) !=
@@ -1112,7 +1347,6 @@ int route_split(int T, int N, int d, int mode, int num_sms) {
   if (route_recv_bytes(L.b_rows) > L.stages * L.stage_bytes) return 1;
   for (int s = kMaxSplit; s > 1; s >>= 1) {
     if (N % s != 0 || (N / s) % 16 != 0 || KB % s != 0 || tiles * s > num_sms) continue;
-    if (mode == kModePredict && route_by_warps(N, s) && route_finish_rows(L, s) < 2) continue;
     if (max_active_clusters(mode, s, N) < tiles) continue;  // must fit in one wave
     return s;
   }
