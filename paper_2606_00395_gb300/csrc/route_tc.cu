@@ -11,34 +11,41 @@
 // tcgen05.mma costs the same issue time for any N <= 256 (one M=128 x N x K=16 step), so a lone
 // tile's chain of d/16 MMAs, not bandwidth, bounds it, and only a K split shortens that chain:
 // CTA r multiplies K blocks [r KB/S, (r+1) KB/S) into a partial [128 x NB] fp32 accumulator
-// (NB = 2N columns [p_old | b] for predict, N for replay).  When the tiles outnumber the SMs
+// (NB = 2N columns [p_old | b] for predict, N for replay and loss).  The widest split whose
+// clusters are all resident at once is taken, for any N and any number of K blocks: when it had
+// to divide them (and N into sixteens) predict of 1000 tokens, d = 2048, took 25.3 us with N = 80
+// (now 9.6), 35.9 with N = 144 (13.1), 26 with N = 256 (17.5), 53.7 with N = 256 and d = 7168
+// (24.8), 29 with N = 128 and d = 2112 (11.5); loss T = 600, N = 160 28.3 (16).  With S = 2 and
+// N > 128 predict splits the two passes over K instead (below).  When the tiles outnumber the SMs
 // (S = 1), each CTA takes half the pipeline stages so that two run on an SM side by side, one
-// CTA's loads and finishing overlapping the other's MMAs (RouteTcArgs::compact).
+// CTA's loads and finishing overlapping the other's MMAs (RouteTcArgs::compact; predict T = 32768,
+// N = 128, d = 2048 51.7 us against 61.8 with one CTA per SM and rows by warps).
 //
 // Warp roles: warp 0 = TMA producer, warp 1 = TMEM owner and MMA issuer, warps 2..5 = epilogue
 // (by warps, below: all sixteen).
 // With S > 1 the partials are reduce-scattered by rows through distributed shared memory: CTA q
 // receives rows [q 128/S, (q+1) 128/S) of every CTA's partial, stored [source][column/4][row][4]
-// so that each warp store moves contiguous bytes; rows beyond the batch are not moved.  Two ways
+// so that each warp store moves contiguous bytes, in as many rounds of columns as shared memory
+// asks for (predict: two or three from N = 176 on); rows beyond the batch are not moved.  Two ways
 // to finish the rows:
-//  - by warps (N <= 128, S >= 4; CTAs of sixteen warps): the warps sum the S copies once, in source
-//    order (deterministic), into rows of shared memory, and each then finishes kRows whole rows, a
-//    lane holding four experts.  predict: the top k + 1 come out one by one by warp maxima
-//    (redux.sync) over orderable 32-bit values.  loss: the dKL/dz rows leave transposed through
-//    shared memory.  Short chains of ALU work per element bound this, not the shuffles or
-//    reductions, so it is the number of warps that counts: calls by threads / six warps / sixteen,
-//    N = 128: predict T = 4001 16.5 / 16.2 / 13.9 us, T = 600 12.9 / 11.1 / 10.3; loss T_c = 2048
-//    18.9 / 21.1 / 17.9; by threads / sixteen warps replay T = 4001 12.4 / 10.4, T = 256 8.9 / 7.5;
-//    predict with N = 64, T = 4096 11.1 / 9.6.
-//  - by threads (everything else): the four epilogue warps sum the S copies in place, walking
-//    consecutive 16-byte words so that no two lanes of a warp hit one bank.  Each row is then
-//    finished by S consecutive threads, thread `part` owning experts [part N/S, (part+1) N/S);
-//    with S = 1 one thread finishes its row straight from TMEM.  A thread reduces its experts to
-//    a max, a sum of exp(z - max) and (predict) its top-16 by 64-bit keys (orderable z bits,
-//    inverted expert index: z descending, ties to the lower expert), built by bitonic sorting 16
-//    experts at a time and merging, in one pass with a running (online) softmax sum; the S
-//    threads of a row then combine max and sum (sum_q s_q exp(m_q - max), fixed shuffle order)
-//    and merge their lists by shuffles.
+//  - by warps (CTAs of sixteen warps; all but the next line): the warps bring the rows into row
+//    order in shared memory, summing the S copies once, in source order (deterministic), and each
+//    then finishes whole rows, a lane holding 2, 4 or 8 experts (N <= 64, 128, 256).  predict: the
+//    top k + 1 come out one by one by warp maxima (redux.sync) over orderable 32-bit values.
+//    loss: the dKL/dz rows leave transposed through shared memory.  Short chains of ALU work per
+//    element bound this, not the shuffles or reductions, so it is the number of warps that counts:
+//    calls by threads / six warps / sixteen, N = 128: predict T = 4001 16.5 / 16.2 / 14.0 us,
+//    T = 600 12.9 / 11.1 / 10.2; loss T_c = 2048 18.9 / 21.1 / 17.7; by threads / sixteen warps
+//    replay T = 4001 12.4 / 10.6, T = 256 9.2 / 7.5; predict T = 4096, N = 64 11.1 / 9.2, T = 8192
+//    (S = 2) 22.2 / 20.5, T = 7000, N = 64, S = 2 13.4 / 12.9 (14.1 with four experts per lane);
+//    S = 1: predict N = 256, T = 12000 46.7 / 44.5, loss T_c = 12000 54.3 / 52.4.
+//  - by threads (predict and replay with S = 1 and N <= 128, or two CTAs per SM): one of 128
+//    threads finishes its row straight from TMEM, without the pass through shared memory (predict
+//    N = 64, T = 15000 25.7 us against 28.6 by warps; replay N = 256 with two CTAs per SM T = 40000
+//    80.3 against 81.9 with one and rows by warps).  It reduces its experts to a max, a sum of
+//    exp(z - max) and (predict) its top-16 by 64-bit keys (orderable z bits, inverted expert
+//    index: z descending, ties to the lower expert), built by bitonic sorting 16 experts at a time
+//    and merging, in one pass with a running (online) softmax sum.
 // Selection is on z in fp32 (softmax is monotone, so the order equals the order of rho_hat).
 #include <float.h>
 
@@ -50,8 +57,8 @@
 namespace pr2 {
 namespace {
 
-constexpr int kThreads = 192;
-constexpr int kWarpThreads = 512;                // CTAs whose rows are finished by warps
+constexpr int kThreads = 192;                    // split = 1
+constexpr int kWarpThreads = 512;                // split > 1: rows finished by warps
 constexpr int kBK = 64;                          // bf16 elements per 128-byte swizzle row
 constexpr int kATileBytes = kTileM * kBK * 2;    // 16 KB
 constexpr int kKeep = kMaxTopK + 1;              // top-(k+1) kept for the margin
@@ -60,19 +67,24 @@ static_assert(kMaxSplit == kRouteMaxSplit, "histogram rows per routing tile");
 constexpr int kMaxStages = 12;
 constexpr int kStageBudget = 192 * 1024;    // pipeline stages of a CTA alone on its SM
 constexpr int kCompactBudget = 96 * 1024;   // two CTAs per SM (more token tiles than SMs)
+constexpr int kFinishBudget = 224 * 1024;   // exchange and finishing of a CTA alone on its SM
 
 struct RouteSmemLayout {
   int stages;
-  int b_rows;        // rows of the weight tile: 2N (predict) or N (replay)
+  int b_rows;        // rows of the weight tile: 2N (predict) or N (replay, loss)
   int passes;        // passes over K: 2 streams [W] then [W_p] (predict, N > 128), else 1
   int pass_rows;     // weight rows of a stage: b_rows / passes
   int stage_bytes;   // A + B
-  int bar_offset;    // after all stages
+  int acc_cols;      // accumulator columns of a CTA (pass split: those of one pass)
+  int xcols;         // split > 1: columns of a partial row that one round of the exchange moves
+  int frows;         // rows finished at once: all 128 / S, or (S = 1, N > 208) half of them
+  int bar_offset;    // after all stages (and after what the exchange and the rows take)
   int total;         // dynamic smem bytes requested (incl. 1 KB alignment slack)
 };
 
-__host__ __device__ inline RouteSmemLayout route_layout(int N, bool predict, bool compact) {
+__host__ __device__ inline RouteSmemLayout route_layout(int N, int mode, int split, bool compact) {
   RouteSmemLayout L;
+  const bool predict = mode == kModePredict;
   L.b_rows = predict ? 2 * N : N;
   // Predict with more than 128 experts: [W; W_p] would make 80 KB stages (two in flight at
   // most), so the router and the predictor weights stream in two passes over K instead, each
@@ -84,22 +96,21 @@ __host__ __device__ inline RouteSmemLayout route_layout(int N, bool predict, boo
   if (L.stages > kMaxStages) L.stages = kMaxStages;
   if (L.stages < 2) L.stages = 2;
   L.bar_offset = L.stages * L.stage_bytes;
+  L.acc_cols = L.passes == 2 && split == 2 ? N : L.b_rows;
+  L.xcols = split > 1 ? L.acc_cols : 0;
+  L.frows = kTileM / split;
+  if (!compact) {
+    // After the K blocks the stages' bytes hold the received copies [S][xcols/4][128/S][4] fp32,
+    // in as few rounds as fit, then the rows in row order (loss: and as bf16).
+    const int row = (L.b_rows / 4 + 1) * 16 + (mode == kModeLoss ? N * 2 + 8 : 0);
+    while (L.frows * row > kFinishBudget) L.frows /= 2;
+    for (int n = 2; L.xcols * kTileM * 4 + L.frows * row > kFinishBudget; ++n)
+      L.xcols = ((L.acc_cols + n - 1) / n + 15) & ~15;
+    const int need = L.xcols * kTileM * 4 + L.frows * row;
+    if (need > L.bar_offset) L.bar_offset = (need + 15) & ~15;
+  }
   L.total = 1024 + L.bar_offset + 256;
   return L;
-}
-
-// Bytes of the reduce-scatter buffer, [S][NB/S/4][128][4] fp32, placed over the pipeline
-// stages once every CTA of the cluster has finished its K blocks.
-__host__ __device__ inline int route_recv_bytes(int b_rows) { return b_rows * kTileM * 4; }
-
-// Whether rows are finished by warps.
-__host__ __device__ inline bool route_by_warps(int N, int split) {
-  return N <= 128 && split >= 4;
-}
-// Shared memory that this takes: the received copies, the rows in row order and (loss) bf16 rows.
-__host__ __device__ inline int route_warps_bytes(const RouteSmemLayout& L, int split) {
-  const int rows = kTileM / split;
-  return route_recv_bytes(L.b_rows) + rows * ((L.b_rows / 4 + 1) * 16 + L.b_rows * 2 + 8);
 }
 
 __host__ __device__ inline uint32_t tmem_cols_for(int cols) {
@@ -201,6 +212,34 @@ __device__ __forceinline__ uint32_t order_bits(float z) {
 __device__ __forceinline__ float order_value(uint32_t ord) {
   return __uint_as_float((ord & 0x80000000u) ? (ord & 0x7fffffffu) : ~ord);
 }
+// kE floats of shared or global memory from p (aligned to their size, at most 16 bytes).
+template <int kE>
+__device__ __forceinline__ void load_vec(const float* p, float (&v)[kE]) {
+  if constexpr (kE == 2) {
+    const float2 x = *reinterpret_cast<const float2*>(p);
+    v[0] = x.x;
+    v[1] = x.y;
+  } else {
+#pragma unroll
+    for (int q = 0; q < kE; q += 4) {
+      const float4 x = *reinterpret_cast<const float4*>(p + q);
+      v[q] = x.x;
+      v[q + 1] = x.y;
+      v[q + 2] = x.z;
+      v[q + 3] = x.w;
+    }
+  }
+}
+template <int kE>
+__device__ __forceinline__ void store_vec(float* p, const float (&v)[kE]) {
+  if constexpr (kE == 2) {
+    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+  } else {
+#pragma unroll
+    for (int q = 0; q < kE; q += 4)
+      *reinterpret_cast<float4*>(p + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+  }
+}
 // Warp-wide operations on kRB rows at once: a warp issues in order, so each step is written for all
 // rows before the next one.
 template <int kRB>
@@ -220,51 +259,53 @@ __device__ __forceinline__ void warp_max(uint32_t (&v)[kRB]) {
   for (int j = 0; j < kRB; ++j) v[j] = __reduce_max_sync(0xffffffffu, v[j]);
 }
 
-// Finishes kRB predict rows by one warp (N <= 128).  Row j: [p_old | b] of 2 N floats at rows[j] in
-// shared memory, token t[j] (live[j]: inside the batch).  Lane l holds experts 4 l .. 4 l + 3,
+// Finishes kRB predict rows by one warp (N <= 32 kE).  Row j: [p_old | b] of 2 N floats at rows[j] in
+// shared memory, token t[j] (live[j]: inside the batch).  Lane l holds experts kE l .. kE l + kE - 1,
 // sorted once; the top k + 1 then come out one by one, the lane whose head equals the warp's
 // maximum giving it (the lowest such lane: z descending, ties to the lower expert).  Writes p_old,
 // idx, gates (divided by their sum under PR2_F_NORMALIZE_TOPK), counts the experts into `hist`
 // (with `count`) and returns the number of rows with rho_hat_(k) - rho_hat_(k+1) <
 // PR2_NEAR_TIE_GAP, always on the unnormalised probabilities.
-template <int kRB>
-__device__ __forceinline__ int finish_predict_rows(const float4* const (&rows)[kRB],
+template <int kRB, int kE>
+__device__ __forceinline__ int finish_predict_rows(const float* const (&rows)[kRB],
                                                    const int64_t (&t)[kRB],
                                                    const bool (&live)[kRB], const RouteTcArgs& a,
                                                    bool count, int (&hist)[kMaxExperts]) {
   const int lane = threadIdx.x & 31;
-  const int n4 = a.N / 4;
-  uint32_t key[kRB][4];
+  const bool in = lane * kE < a.N;
+  uint32_t key[kRB][kE];
   uint32_t ids[kRB];  // the lane's experts in the order of its keys, 4 bits each
   uint32_t head[kRB];
-  float mx[kRB], sum[kRB], my_z[kRB], zs[kRB][4];
+  float mx[kRB], sum[kRB], my_z[kRB], zs[kRB][kE];
   int my_e[kRB];
 #pragma unroll
   for (int j = 0; j < kRB; ++j) {
-    float z[4];
-    if (lane < n4) {
-      const float4 p = rows[j][lane], b = rows[j][n4 + lane];
-      if (a.logits_or_probs != nullptr && live[j])
-        reinterpret_cast<float4*>(a.logits_or_probs + t[j] * a.N)[lane] = p;
-      z[0] = p.x + b.x;
-      z[1] = p.y + b.y;
-      z[2] = p.z + b.z;
-      z[3] = p.w + b.w;
+    float z[kE];
+    uint32_t id[kE];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) key[j][q] = order_bits(z[q]);
+    for (int q = 0; q < kE; ++q) id[q] = q;
+    if (in) {
+      float b[kE];
+      load_vec<kE>(rows[j] + lane * kE, z);
+      load_vec<kE>(rows[j] + a.N + lane * kE, b);
+      if (a.logits_or_probs != nullptr && live[j])
+        store_vec<kE>(a.logits_or_probs + t[j] * a.N + lane * kE, z);
+#pragma unroll
+      for (int q = 0; q < kE; ++q) z[q] += b[q];
+#pragma unroll
+      for (int q = 0; q < kE; ++q) key[j][q] = order_bits(z[q]);
     } else {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < kE; ++q) {
         z[q] = -INFINITY;
         key[j][q] = 0u;
       }
     }
-    uint32_t id[4] = {0u, 1u, 2u, 3u};
     // odd-even transposition: neighbours swap only when out of order, so equal values keep theirs
 #pragma unroll
-    for (int ph = 0; ph < 4; ++ph)
+    for (int ph = 0; ph < kE; ++ph)
 #pragma unroll
-      for (int q = ph & 1; q + 1 < 4; q += 2) {
+      for (int q = ph & 1; q + 1 < kE; q += 2) {
         const bool sw = key[j][q + 1] > key[j][q];
         const uint32_t k0 = key[j][q], i0 = id[q];
         key[j][q] = sw ? key[j][q + 1] : k0;
@@ -272,10 +313,12 @@ __device__ __forceinline__ int finish_predict_rows(const float4* const (&rows)[k
         id[q] = sw ? id[q + 1] : i0;
         id[q + 1] = sw ? i0 : id[q + 1];
       }
-    ids[j] = id[0] | id[1] << 4 | id[2] << 8 | id[3] << 12;
+    ids[j] = 0u;
+#pragma unroll
+    for (int q = 0; q < kE; ++q) ids[j] |= id[q] << (4 * q);
     head[j] = key[j][0];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) zs[j][q] = z[q];
+    for (int q = 0; q < kE; ++q) zs[j][q] = z[q];
     my_z[j] = 0.f;
     my_e[j] = 0;
   }
@@ -284,9 +327,9 @@ __device__ __forceinline__ int finish_predict_rows(const float4* const (&rows)[k
   for (int j = 0; j < kRB; ++j) {
     mx[j] = fmaxf(order_value(head[j]), -FLT_MAX);
     sum[j] = 0.f;
-    if (lane < n4)
+    if (in)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) sum[j] += expf(zs[j][q] - mx[j]);
+      for (int q = 0; q < kE; ++q) sum[j] += expf(zs[j][q] - mx[j]);
   }
   warp_add<kRB>(sum);
   const int rounds = a.k < a.N ? a.k + 1 : a.k;
@@ -302,17 +345,17 @@ __device__ __forceinline__ int finish_predict_rows(const float4* const (&rows)[k
     for (int j = 0; j < kRB; ++j) has[j] = __ballot_sync(0xffffffffu, key[j][0] == head[j]);
 #pragma unroll
     for (int j = 0; j < kRB; ++j)
-      e[j] = __shfl_sync(0xffffffffu, lane * 4 + static_cast<int>(ids[j] & 15u), __ffs(has[j]) - 1);
+      e[j] = __shfl_sync(0xffffffffu, lane * kE + static_cast<int>(ids[j] & 15u), __ffs(has[j]) - 1);
 #pragma unroll
     for (int j = 0; j < kRB; ++j) {
       if (lane == r) {
         my_z[j] = order_value(head[j]);
         my_e[j] = e[j];
       }
-      if (lane == e[j] >> 2) {
+      if (lane == e[j] / kE) {
 #pragma unroll
-        for (int q = 0; q < 3; ++q) key[j][q] = key[j][q + 1];
-        key[j][3] = 0u;
+        for (int q = 0; q < kE - 1; ++q) key[j][q] = key[j][q + 1];
+        key[j][kE - 1] = 0u;
         ids[j] >>= 4;
       }
     }
@@ -342,33 +385,44 @@ __device__ __forceinline__ int finish_predict_rows(const float4* const (&rows)[k
 }
 
 // kRB replay rows finished by one warp: row j's logits are N floats at rows[j] (lane l: experts
-// 4 l ..), lane s < k holds cached slot s in es[j] (-1: none, out of range or repeated).  Writes
+// kE l ..), lane s < k holds cached slot s in es[j] (-1: none, out of range or repeated).  Writes
 // the gates (divided by their sum over the valid slots under PR2_F_NORMALIZE_TOPK) and, where
 // asked for, the row of rho.
-template <int kRB>
-__device__ __forceinline__ void finish_replay_rows(const float4* const (&rows)[kRB],
+template <int kRB, int kE>
+__device__ __forceinline__ void finish_replay_rows(const float* const (&rows)[kRB],
                                                    const int (&es)[kRB], const int64_t (&t)[kRB],
                                                    const bool (&live)[kRB], const RouteTcArgs& a) {
   const int lane = threadIdx.x & 31;
-  const int n4 = a.N / 4;
-  float4 z[kRB];
+  const bool in = lane * kE < a.N;
+  float z[kRB][kE];
   uint32_t head[kRB];
   float sum[kRB], g[kRB], sk[kRB];
 #pragma unroll
   for (int j = 0; j < kRB; ++j) {
-    z[j] = lane < n4 ? rows[j][lane] : make_float4(-FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX);
-    head[j] = order_bits(fmaxf(fmaxf(z[j].x, z[j].y), fmaxf(z[j].z, z[j].w)));
+    float c = -FLT_MAX;
+    if (in) {
+      load_vec<kE>(rows[j] + lane * kE, z[j]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < kE; ++q) z[j][q] = -FLT_MAX;
+    }
+#pragma unroll
+    for (int q = 0; q < kE; ++q) c = fmaxf(c, z[j][q]);
+    head[j] = order_bits(c);
   }
   warp_max<kRB>(head);
 #pragma unroll
   for (int j = 0; j < kRB; ++j) {
     const float mx = fmaxf(order_value(head[j]), -FLT_MAX);
-    const float zg = es[j] >= 0 ? reinterpret_cast<const float*>(rows[j])[es[j]] : 0.f;
-    z[j].x = expf(z[j].x - mx);
-    z[j].y = expf(z[j].y - mx);
-    z[j].z = expf(z[j].z - mx);
-    z[j].w = expf(z[j].w - mx);
-    sum[j] = lane < n4 ? (z[j].x + z[j].y) + (z[j].z + z[j].w) : 0.f;
+    const float zg = es[j] >= 0 ? rows[j][es[j]] : 0.f;
+    float part = 0.f;
+#pragma unroll
+    for (int q = 0; q < kE; q += 2) {
+      z[j][q] = expf(z[j][q] - mx);
+      z[j][q + 1] = expf(z[j][q + 1] - mx);
+      part += z[j][q] + z[j][q + 1];
+    }
+    sum[j] = in ? part : 0.f;
     g[j] = es[j] >= 0 ? expf(zg - mx) : 0.f;
   }
   warp_add<kRB>(sum);
@@ -379,40 +433,49 @@ __device__ __forceinline__ void finish_replay_rows(const float4* const (&rows)[k
   for (int j = 0; j < kRB; ++j) {
     if (!live[j]) continue;
     if (lane < a.k) a.gates[t[j] * a.k + lane] = a.norm && sk[j] > 0.f ? g[j] * (1.0f / sk[j]) : g[j];
-    if (a.logits_or_probs != nullptr && lane < n4) {
+    if (a.logits_or_probs != nullptr && in) {
       const float inv = 1.0f / sum[j];
-      reinterpret_cast<float4*>(a.logits_or_probs + t[j] * a.N)[lane] =
-          make_float4(z[j].x * inv, z[j].y * inv, z[j].z * inv, z[j].w * inv);
+#pragma unroll
+      for (int q = 0; q < kE; ++q) z[j][q] *= inv;
+      store_vec<kE>(a.logits_or_probs + t[j] * a.N + lane * kE, z[j]);
     }
   }
 }
 
-// The loss mode's rows finished by one warp, kRB at a time: row j's predictor logits b are N floats
-// at rows[j] (lane l: experts 4 l ..), its p_old and teacher values po[j], tr[j].  Writes the
-// per-token KL and the bf16 dKL/dz row to gs[j] (shared memory); formulas at the thread-wise form
-// in the kernel.
-template <int kRB>
-__device__ __forceinline__ void finish_loss_rows(const float4* const (&rows)[kRB],
-                                                 const float4 (&po4)[kRB], const float4 (&tr4)[kRB],
+// kRB rows of the predictive loss (Eq. pr2_loss, Algorithm 3) finished by one warp: row j's
+// predictor logits b are N floats at rows[j] (lane l: experts kE l ..), its p_old and teacher
+// values (row pos[t] of rho) po[j], tr[j]:
+//   standard: prediction Softmax(v), v = p_old + b;  target rho
+//   delta:    prediction Softmax(b);  target Softmax(u), u = log rho - p_old
+// KL_t = sum_j tgt_j (log tgt_j - log pred_j);  dKL_t/dv_j = pred_j - tgt_j, rounded to bf16 and
+// written to gs[j] (shared memory).  Exponentials and logarithms use the hardware approximations
+// (__expf, __logf: a few ulp over the ranges met here, far inside the loss's tolerance).
+template <int kRB, int kE>
+__device__ __forceinline__ void finish_loss_rows(const float* const (&rows)[kRB],
+                                                 const float (&po)[kRB][kE],
+                                                 const float (&tr)[kRB][kE],
                                                  const bool (&use)[kRB], const int64_t (&t)[kRB],
-                                                 uint2* const (&gs)[kRB], const RouteTcArgs& a) {
+                                                 uint32_t* const (&gs)[kRB], const RouteTcArgs& a) {
   const int lane = threadIdx.x & 31;
-  const bool delta = a.delta != 0, in = lane < a.N / 4;
-  float v[kRB][4], lt[kRB][4], tg[kRB][4], s1[kRB], s2[kRB], kl[kRB];
+  const bool delta = a.delta != 0, in = lane * kE < a.N;
+  float v[kRB][kE], lt[kRB][kE], tg[kRB][kE], s1[kRB], s2[kRB], kl[kRB];
   uint32_t m1[kRB], m2[kRB];  // row maxima (order_bits: no NaN among the candidates)
 #pragma unroll
   for (int j = 0; j < kRB; ++j) {
-    const float4 b4 = in ? rows[j][lane] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float b[4] = {b4.x, b4.y, b4.z, b4.w};
-    const float po[4] = {po4[j].x, po4[j].y, po4[j].z, po4[j].w};
-    const float tr[4] = {tr4[j].x, tr4[j].y, tr4[j].z, tr4[j].w};
     float c1 = -FLT_MAX, c2 = -FLT_MAX;
+    float b[kE];
+    if (in) {
+      load_vec<kE>(rows[j] + lane * kE, b);
+    } else {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < kE; ++q) b[q] = 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < kE; ++q) {
       const bool ok = in && use[j];
-      v[j][q] = ok ? (delta ? b[q] : po[q] + b[q]) : -INFINITY;
-      tg[j][q] = ok ? tr[q] : 0.f;
-      lt[j][q] = ok && tr[q] > 0.f ? __logf(tr[q]) - (delta ? po[q] : 0.f) : -INFINITY;
+      v[j][q] = ok ? (delta ? b[q] : po[j][q] + b[q]) : -INFINITY;
+      tg[j][q] = ok ? tr[j][q] : 0.f;
+      lt[j][q] = ok && tr[j][q] > 0.f ? __logf(tr[j][q]) - (delta ? po[j][q] : 0.f) : -INFINITY;
       c1 = fmaxf(c1, v[j][q]);
       c2 = fmaxf(c2, lt[j][q]);
     }
@@ -425,7 +488,7 @@ __device__ __forceinline__ void finish_loss_rows(const float4* const (&rows)[kRB
   for (int j = 0; j < kRB; ++j) {
     s1[j] = s2[j] = 0.f;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < kE; ++q) {
       s1[j] += __expf(v[j][q] - order_value(m1[j]));
       if (delta) s2[j] += __expf(lt[j][q] - order_value(m2[j]));
     }
@@ -436,17 +499,19 @@ __device__ __forceinline__ void finish_loss_rows(const float4* const (&rows)[kRB
   for (int j = 0; j < kRB; ++j) {
     const float l1 = order_value(m1[j]) + __logf(s1[j]);  // log normalisers
     const float l2 = delta ? order_value(m2[j]) + __logf(s2[j]) : 0.f;
-    float g[4];
+    float g[kE];
     kl[j] = 0.f;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < kE; ++q) {
       const float lp = v[j][q] - l1;  // log prediction
       const float ltq = lt[j][q] - l2;
       const float tgt = delta ? (tg[j][q] > 0.f ? __expf(ltq) : 0.f) : tg[j][q];
       if (tgt > 0.f) kl[j] += tgt * (ltq - lp);
       g[q] = in && use[j] ? __expf(lp) - tgt : 0.f;
     }
-    if (in) *gs[j] = make_uint2(pack_bf16x2(g[0], g[1]), pack_bf16x2(g[2], g[3]));
+    if (in)
+#pragma unroll
+      for (int q = 0; q < kE; q += 2) gs[j][q / 2] = pack_bf16x2(g[q], g[q + 1]);
   }
   warp_add<kRB>(kl);
 #pragma unroll
@@ -454,16 +519,18 @@ __device__ __forceinline__ void finish_loss_rows(const float4* const (&rows)[kRB
     if (lane == 0 && t[j] < a.T) a.kl_tok[t[j]] = use[j] ? kl[j] : 0.f;
 }
 
-template <int kMode, int split, bool by_warps>
-__global__ void __launch_bounds__(by_warps ? kWarpThreads : kThreads, 1)
+// kE: experts of a lane where rows are finished by warps (2, 4 or 8: N <= 32 kE); 0: by threads.
+template <int kMode, int split, int kE>
+__global__ void __launch_bounds__(kE > 0 ? kWarpThreads : kThreads, 1)
     route_tc_kernel(const __grid_constant__ CUtensorMap tm_h,
                     const __grid_constant__ CUtensorMap tm_w,
                     const __grid_constant__ CUtensorMap tm_wp, RouteTcArgs a) {
   constexpr bool predict = kMode == kModePredict;
   constexpr bool loss = kMode == kModeLoss;
+  constexpr bool by_warps = kE > 0;
   extern __shared__ __align__(16) uint8_t smem_raw[];
   const int N = a.N, k = a.k;
-  const RouteSmemLayout L = route_layout(N, predict, a.compact != 0);
+  const RouteSmemLayout L = route_layout(N, kMode, split, a.compact != 0);
   // 1024-B aligned base, kept as an offset into the shared array so the compiler knows every
   // derived pointer is shared memory.
   const uint32_t pad = (1024u - (smem_u32(smem_raw) & 1023u)) & 1023u;
@@ -474,26 +541,22 @@ __global__ void __launch_bounds__(by_warps ? kWarpThreads : kThreads, 1)
   uint64_t* drain = acc_full + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  const float4* recv = reinterpret_cast<const float4*>(smem);  // valid after the exchange
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int rank = split > 1 ? static_cast<int>(cluster_ctarank()) : 0;
   const int t0 = (blockIdx.x / split) * kTileM;
-  const int R = kTileM / split;             // rows finished by this CTA
-  const int nr = N / split;                 // experts of one finishing thread
   const int nb4 = L.b_rows / 4;             // float4 columns of a partial row
   // Pass split: predict whose weights stream in two passes (N > 128) run by a 2-CTA cluster in
   // which CTA r streams pass r ([W], then [W_p]) over all of K; the two column halves of every
-  // row then meet in the CTA that finishes it, through distributed shared memory, and are not
-  // summed.  Otherwise the cluster splits K and the S partial rows are summed.
+  // row then meet in the CTA that finishes it and are not summed: half the exchange of a K split.
   const bool psplit = predict && L.passes == 2 && split == 2;
-  const int KBper = psplit ? a.d / kBK : (a.d / kBK) / split;
-  const int kb0 = psplit ? 0 : rank * KBper, kb1 = kb0 + KBper;
+  const int KB = a.d / kBK;                 // K blocks, of which this CTA takes [kb0, kb1)
+  const int kb0 = psplit ? 0 : rank * KB / split;
+  const int kb1 = psplit ? KB : (rank + 1) * KB / split;
   const int npass = psplit ? 1 : L.passes;  // passes this CTA streams
   const int pass0 = psplit ? rank : 0;      // the first of them
-  const int acc_cols = psplit ? L.pass_rows : L.b_rows;
-  const uint32_t ncols = tmem_cols_for(acc_cols);
+  const uint32_t ncols = tmem_cols_for(L.acc_cols);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < L.stages; ++s) {
@@ -613,19 +676,14 @@ __global__ void __launch_bounds__(by_warps ? kWarpThreads : kThreads, 1)
   // predict: experts of the rows this CTA finishes, for the dispatch that follows
   __shared__ int hist_s[kMaxExperts];
   const bool count = predict && a.hist != nullptr;
-  if (count && epi) {  // (split > 1: the cluster barriers below order it before the counting)
+  if (count && epi) {  // (by warps: the barriers below order it before the counting)
     for (int e = threadIdx.x - 64; e < N; e += 128) hist_s[e] = 0;
-    if (split == 1) named_bar_sync(1, 128);
+    if (!by_warps) named_bar_sync(1, 128);
   }
   const int q = warp & 3;
   const int row = q * 32 + lane;  // TMEM lane of this thread
   const uint32_t trow = tmem + (static_cast<uint32_t>(q * 32) << 16);
-  // Finishing coordinates: row lr of this CTA's R rows, experts [part nr, (part+1) nr).
-  const int et = threadIdx.x - 64;
-  const int lr = split == 1 ? row : et / split;
-  const int part = split == 1 ? 0 : et - lr * split;
-  const int fe0 = part * nr;
-  const int64_t t = static_cast<int64_t>(t0) + static_cast<int64_t>(rank) * R + lr;
+  const int64_t t = static_cast<int64_t>(t0) + row;  // split = 1: this thread's row
   const bool live = epi && t < a.T;
 
   // replay: cached indices, validated (range, duplicates) while the K blocks run
@@ -650,197 +708,207 @@ __global__ void __launch_bounds__(by_warps ? kWarpThreads : kThreads, 1)
     }
   }
 
-  // loss: the first kLossPre experts of this thread's segment of its p_old row and of its
-  // teacher row (row pos[t] of rho), loaded while the K blocks run
-  constexpr int kLossPre = loss ? 32 : 4;
-  float po_s[kLossPre], tr_s[kLossPre];
-  int64_t lrow = 0;
-  bool okp = false;
-  // finished by warps: this warp's rows wr0 .. wr0 + kRows - 1 of the CTA's; loss: their p_old and
-  // teacher values (row pos[t] of rho), loaded while the K blocks run
-  constexpr int kRows = by_warps ? kTileM / split / (kWarpThreads / 32) : 1;
-  static_assert(!by_warps || kRows * split * (kWarpThreads / 32) == kTileM, "whole rows per warp");
-  const int wr0 = warp * kRows;
-  const int64_t tw = static_cast<int64_t>(t0) + static_cast<int64_t>(rank) * R + wr0;
-  float4 po_w[kRows], tr_w[kRows];
-  bool use_w[kRows];
-  int es_w[kRows];  // replay: cached slot `lane` of the row, -1 if it does not count
-  if (kMode == kModeReplay && by_warps) {
-    bool wrong = false;
+  // finished by warps: the CTA's kR rows, frows of them at once, fper of those by each warp, kRB
+  // at a time; replay: cached slot `lane` of each row, -1 if it does not count; loss: p_old and
+  // teacher values (row pos[t] of rho).  The first kRB rows' are loaded while the K blocks run.
+  constexpr int kR = kTileM / split;
+  constexpr int kRows = kR / (kWarpThreads / 32);
+  constexpr int kLane = by_warps ? kE : 2;
+  constexpr int kHeld = loss && split < 4 ? 8 : 16;  // logits a lane holds at once (registers)
+  constexpr int kRB = kRows * kLane > kHeld ? kHeld / kLane : kRows;
+  const int frows = split > 1 ? kR : L.frows, fper = split > 1 ? kRows : L.frows / 16;
+  const int64_t tc = static_cast<int64_t>(t0) + rank * kR;  // token of the CTA's row 0
+  float po_w[kRB][kLane], tr_w[kRB][kLane];
+  bool use_w[kRB];
+  int es_w[kRB];
+  auto load_rows = [&](int r0) {  // of the CTA's rows r0 .. r0 + kRB - 1
+    if constexpr (kMode == kModeReplay) {
+      bool wrong = false;
 #pragma unroll
-    for (int j = 0; j < kRows; ++j) {
-      const bool in = tw + j < a.T && lane < k;
-      es_w[j] = in ? a.idx_in[(tw + j) * k + lane] : -1;
-    }
-#pragma unroll
-    for (int j = 0; j < kRows; ++j) {
-      const int e = es_w[j];
-      bool ok = e >= 0 && e < N;
-#pragma unroll
-      for (int s2 = 0; s2 < kMaxTopK - 1; ++s2) {
-        // a repeat counts against its later slot; an entry out of range repeats nothing
-        const int other = __shfl_sync(0xffffffffu, e, s2);
-        if (s2 < lane && other == e) ok = false;
+      for (int j = 0; j < kRB; ++j) {
+        const bool in = tc + r0 + j < a.T && lane < k;
+        es_w[j] = in ? a.idx_in[(tc + r0 + j) * k + lane] : -1;
       }
-      wrong = wrong || (tw + j < a.T && lane < k && !ok);
-      if (!ok) es_w[j] = -1;
-    }
-    if (wrong && a.status != nullptr) atomicOr(a.status, PR2_STATUS_BAD_INDEX);
-  }
-  if (loss && by_warps) {
-    int32_t pw[kRows];
 #pragma unroll
-    for (int j = 0; j < kRows; ++j)
-      pw[j] = tw + j < a.T && a.pos != nullptr ? a.pos[tw + j] : 0;
+      for (int j = 0; j < kRB; ++j) {
+        const int e = es_w[j];
+        bool ok = e >= 0 && e < N;
 #pragma unroll
-    for (int j = 0; j < kRows; ++j) {
-      const int64_t r = a.pos != nullptr ? static_cast<int64_t>(pw[j]) : tw + j;
-      use_w[j] = tw + j < a.T && r >= 0 && r < a.T_rho;
-      if (tw + j < a.T && !use_w[j] && lane == 0 && a.status != nullptr)
-        atomicOr(a.status, PR2_STATUS_BAD_INDEX);
-      po_w[j] = tr_w[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (use_w[j] && lane < N / 4) {
-        po_w[j] = reinterpret_cast<const float4*>(a.p_old + (tw + j) * N)[lane];
-        tr_w[j] = reinterpret_cast<const float4*>(a.rho + r * N)[lane];
+        for (int s2 = 0; s2 < kMaxTopK - 1; ++s2) {
+          // a repeat counts against its later slot; an entry out of range repeats nothing
+          const int other = __shfl_sync(0xffffffffu, e, s2);
+          if (s2 < lane && other == e) ok = false;
+        }
+        wrong = wrong || (tc + r0 + j < a.T && lane < k && !ok);
+        if (!ok) es_w[j] = -1;
       }
+      if (wrong && a.status != nullptr) atomicOr(a.status, PR2_STATUS_BAD_INDEX);
     }
-  }
-  if (loss && live && !by_warps) {
-    lrow = a.pos != nullptr ? static_cast<int64_t>(a.pos[t]) : t;
-    okp = lrow >= 0 && lrow < a.T_rho;
-    if (okp) {
-      const float4* p4 = reinterpret_cast<const float4*>(a.p_old + t * N + fe0);
-      const float4* r4 = reinterpret_cast<const float4*>(a.rho + lrow * N + fe0);
+    if constexpr (loss) {
+      int32_t pw[kRB];
 #pragma unroll
-      for (int j = 0; j < kLossPre / 4; ++j) {
-        if (4 * j < nr) {
-          const float4 x = p4[j], y = r4[j];
-          po_s[4 * j] = x.x;
-          po_s[4 * j + 1] = x.y;
-          po_s[4 * j + 2] = x.z;
-          po_s[4 * j + 3] = x.w;
-          tr_s[4 * j] = y.x;
-          tr_s[4 * j + 1] = y.y;
-          tr_s[4 * j + 2] = y.z;
-          tr_s[4 * j + 3] = y.w;
+      for (int j = 0; j < kRB; ++j)
+        pw[j] = tc + r0 + j < a.T && a.pos != nullptr ? a.pos[tc + r0 + j] : 0;
+#pragma unroll
+      for (int j = 0; j < kRB; ++j) {
+        const int64_t tj = tc + r0 + j;
+        const int64_t r = a.pos != nullptr ? static_cast<int64_t>(pw[j]) : tj;
+        use_w[j] = tj < a.T && r >= 0 && r < a.T_rho;
+        if (tj < a.T && !use_w[j] && lane == 0 && a.status != nullptr)
+          atomicOr(a.status, PR2_STATUS_BAD_INDEX);
+#pragma unroll
+        for (int c = 0; c < kLane; ++c) po_w[j][c] = tr_w[j][c] = 0.f;
+        if (use_w[j] && lane * kLane < N) {
+          load_vec<kLane>(a.p_old + tj * N + lane * kLane, po_w[j]);
+          load_vec<kLane>(a.rho + r * N + lane * kLane, tr_w[j]);
         }
       }
     }
-  }
-
+  };
+  if (by_warps) load_rows(warp * fper);
   bool have = false;
   if (epi || by_warps) {
     // tcgen05.ld is warp-collective: the whole warp reads TMEM or none of it does.
     have = __all_sync(0xffffffffu, mbar_wait(acc_full, 0, abort_flag, a.status));
     if (have) tc_fence_after();
   }
-  if (split > 1) {
-    cluster_sync();  // every CTA has finished its K blocks: the pipeline stages are free
-    if ((epi || by_warps) && have) {
-      // Reduce-scatter by rows: this TMEM row goes to CTA row / R as its row row % R, into the
-      // slot of source `rank` (K split) or into columns [rank N, (rank + 1) N) (pass split).
-      // With sixteen warps the four of a lane quadrant share its columns.
-      float4* recv_w = reinterpret_cast<float4*>(smem);
-      const uint32_t dst = static_cast<uint32_t>(row / R);
-      const int drow = row - static_cast<int>(dst) * R;
-      const int off4 = psplit ? L.pass_rows / 4 : nb4;
-      const uint32_t rbase =
-          mapa_shared(smem_u32(recv_w + (rank * off4) * R + drow), dst);
-      // rows beyond the batch are not moved (a decode batch fills a few rows of its tile); a
-      // warp of such rows skips its loads too
-      const bool in_batch = static_cast<int64_t>(t0) + row < a.T;
-      const int cols = static_cast<int64_t>(t0) + q * 32 < a.T ? acc_cols : 0;
-      constexpr int kShare = by_warps ? kWarpThreads / 128 : 1;
-      for (int c0 = by_warps ? (warp >> 2) * 32 : 0; c0 < cols; c0 += 32 * kShare) {
-        uint32_t r0[16], r1[16];
-        tmem_ld16(trow + c0, r0);
-        tmem_ld16(trow + c0 + 16, r1);
-        tmem_wait_ld(r0);
-        reg_fence(r1);
-        if (!in_batch) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          st_cluster_v4(rbase + static_cast<uint32_t>(((c0 / 4 + j) * R) * 16), r0[4 * j],
-                        r0[4 * j + 1], r0[4 * j + 2], r0[4 * j + 3]);
-        if (c0 + 16 < acc_cols) {  // a multiple of 16, not always of 32
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            st_cluster_v4(rbase + static_cast<uint32_t>(((c0 / 4 + 4 + j) * R) * 16), r1[4 * j],
-                          r1[4 * j + 1], r1[4 * j + 2], r1[4 * j + 3]);
-        }
-      }
-    }
-    cluster_sync();  // every partial row has landed
-    if (epi && !psplit && !by_warps) {
-      // Sum the S received copies of this CTA's rows once, in source order, into source 0's
-      // slots: consecutive threads take consecutive 16-byte words (no bank conflicts), so the
-      // finishing threads then read one value per column instead of S strided ones.
-      float4* red = reinterpret_cast<float4*>(smem);
-      const int n4 = nb4 * R;  // 16-byte words of one source
-      for (int i = threadIdx.x - 64; i < n4; i += 128) {
-        float4 v = red[i];
-#pragma unroll
-        for (int src = 1; src < split; ++src) {
-          const float4 w = red[src * n4 + i];
-          v.x += w.x;
-          v.y += w.y;
-          v.z += w.z;
-          v.w += w.w;
-        }
-        red[i] = v;
-      }
-      named_bar_sync(1, 128);  // the four epilogue warps
-    }
-  }
-  // Columns [c, c + 16) of the finished row: the summed partials (S > 1) or TMEM (S = 1).
+  // Columns [c, c + 16) of this thread's row.
   auto load16 = [&](int c, uint32_t (&r)[16]) {
-    if (split == 1) {
-      tmem_ld16(trow + c, r);
-      tmem_wait_ld(r);
-      return;
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float4 v = recv[(c / 4 + j) * R + lr];
-      r[4 * j] = __float_as_uint(v.x);
-      r[4 * j + 1] = __float_as_uint(v.y);
-      r[4 * j + 2] = __float_as_uint(v.z);
-      r[4 * j + 3] = __float_as_uint(v.w);
-    }
+    tmem_ld16(trow + c, r);
+    tmem_wait_ld(r);
   };
 
   if constexpr (by_warps) {
-    // every thread of the CTA is past the cluster barrier: all sixteen warps sum the S copies into
-    // row order and finish kRows rows each
-    const int pitch4 = nb4 + 1;  // 16-byte words of a row: odd, so 8 rows take 8 bank groups
-    float4* rm = reinterpret_cast<float4*>(smem) + nb4 * kTileM;
-    constexpr int kR = kTileM / split;
-    for (int i = threadIdx.x; i < nb4 * kR; i += kWarpThreads) {
-      float4 v = recv[i];
+    const int pitch = (nb4 + 1) * 4;  // floats of a row: 8 rows in turn take 8 bank groups
+    float4* recv = reinterpret_cast<float4*>(smem);  // [S][columns of a round / 4][kR]
+    float* rm = reinterpret_cast<float*>(smem + L.xcols * kTileM * 4);  // the rows in row order
+    if constexpr (split > 1) {
+      // Reduce-scatter by rows: this TMEM row goes to CTA row / kR as its row row % kR, into the
+      // slot of source `rank`; the four warps of a lane quadrant share its columns.  Rows beyond
+      // the batch are not moved (a decode batch fills a few rows of its tile); a warp of such
+      // rows skips its loads too.
+      const uint32_t dst = static_cast<uint32_t>(row / kR);
+      const bool in_batch = static_cast<int64_t>(t0) + row < a.T;
+      const bool move = have && static_cast<int64_t>(t0) + q * 32 < a.T;
+      for (int x0 = 0; x0 < L.acc_cols; x0 += L.xcols) {
+        const int xn = L.acc_cols - x0 < L.xcols ? L.acc_cols - x0 : L.xcols;
+        cluster_sync();  // every CTA is done with its K blocks (the round before): recv is free
+        if (move) {
+          const uint32_t rbase = mapa_shared(
+              smem_u32(recv + rank * (xn / 4) * kR + (row - static_cast<int>(dst) * kR)), dst);
+          for (int c0 = (warp >> 2) * 32; c0 < xn; c0 += 32 * (kWarpThreads / 128)) {
+            uint32_t r0[16], r1[16];
+            const bool two = c0 + 16 < xn;  // a multiple of 16, not always of 32
+            tmem_ld16(trow + x0 + c0, r0);
+            if (two) tmem_ld16(trow + x0 + c0 + 16, r1);
+            tmem_wait_ld(r0);
+            if (two) reg_fence(r1);
+            if (in_batch) {
 #pragma unroll
-      for (int src = 1; src < split; ++src) {
-        const float4 w = recv[src * nb4 * kR + i];
-        v.x += w.x;
-        v.y += w.y;
-        v.z += w.z;
-        v.w += w.w;
+              for (int j = 0; j < 4; ++j)
+                st_cluster_v4(rbase + static_cast<uint32_t>(((c0 / 4 + j) * kR) * 16), r0[4 * j],
+                              r0[4 * j + 1], r0[4 * j + 2], r0[4 * j + 3]);
+            }
+            if (two && in_batch) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                st_cluster_v4(rbase + static_cast<uint32_t>(((c0 / 4 + 4 + j) * kR) * 16), r1[4 * j],
+                              r1[4 * j + 1], r1[4 * j + 2], r1[4 * j + 3]);
+            }
+          }
+        }
+        cluster_sync();  // every partial row has landed
+        // all sixteen warps bring the copies into row order: summed once, in source order, or
+        // (pass split) source 1's columns behind source 0's
+        const int n4 = (xn / 4) * kR;
+        for (int i = threadIdx.x; i < n4; i += kWarpThreads) {
+          float4 v = recv[i];
+          float4* to = reinterpret_cast<float4*>(rm + (i % kR) * pitch) + x0 / 4 + i / kR;
+          if (psplit) {
+            to[N / 4] = recv[n4 + i];
+          } else {
+#pragma unroll
+            for (int src = 1; src < split; ++src) {
+              const float4 w = recv[src * n4 + i];
+              v.x += w.x;
+              v.y += w.y;
+              v.z += w.z;
+              v.w += w.w;
+            }
+          }
+          *to = v;
+        }
       }
-      rm[(i % kR) * pitch4 + i / kR] = v;
     }
-    __syncthreads();
-    const bool good = *abort_flag == 0;
-    const float4* rows[kRows];
-    int64_t ts[kRows];
-    bool lv[kRows];
+    // the bf16 dKL/dz rows (loss) meet in shared memory
+    uint8_t* gsb = reinterpret_cast<uint8_t*>(rm + frows * pitch);
+    const int gpitch = N * 2 + 8;
+    int ties = 0;
+    for (int f0 = 0; f0 < kR; f0 += frows) {  // rows f0 .. f0 + frows - 1 of the CTA
+      __syncthreads();  // split = 1: every K block, copy and earlier row is done with the stages
+      if constexpr (split == 1) {
+        if (have && row >= f0 && row < f0 + frows) {  // whole warps: frows is 64 or 128
+          float4* to = reinterpret_cast<float4*>(rm + (row - f0) * pitch);
+          for (int c0 = (warp >> 2) * 16; c0 < L.b_rows; c0 += 16 * (kWarpThreads / 128)) {
+            uint32_t r[16];
+            tmem_ld16(trow + c0, r);
+            tmem_wait_ld(r);
 #pragma unroll
-    for (int j = 0; j < kRows; ++j) {
-      rows[j] = rm + (wr0 + j) * pitch4;
-      ts[j] = tw + j;
-      lv[j] = good && ts[j] < a.T;
+            for (int j = 0; j < 4; ++j)
+              to[c0 / 4 + j] =
+                  make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
+                              __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
+          }
+        }
+        __syncthreads();
+      }
+      const bool good = *abort_flag == 0;
+      for (int j0 = 0; j0 < fper; j0 += kRB) {
+        const int fr = warp * fper + j0;  // of the frows rows in shared memory
+        if (f0 > 0 || j0 > 0) load_rows(f0 + fr);
+        const float* rows[kRB];
+        int64_t ts[kRB];
+        bool lv[kRB];
+#pragma unroll
+        for (int j = 0; j < kRB; ++j) {
+          rows[j] = rm + (fr + j) * pitch;
+          ts[j] = tc + f0 + fr + j;
+          lv[j] = good && ts[j] < a.T;
+        }
+        if constexpr (predict) {
+          if (good && ts[0] < a.T)
+            ties += finish_predict_rows<kRB, kLane>(rows, ts, lv, a, count, hist_s);
+        } else if constexpr (kMode == kModeReplay) {
+          if (ts[0] < a.T) finish_replay_rows<kRB, kLane>(rows, es_w, ts, lv, a);
+        } else {
+          uint32_t* gs[kRB];
+#pragma unroll
+          for (int j = 0; j < kRB; ++j) {
+            gs[j] = reinterpret_cast<uint32_t*>(gsb + (fr + j) * gpitch + lane * (kLane * 2));
+            use_w[j] = use_w[j] && good;
+          }
+          finish_loss_rows<kRB, kLane>(rows, po_w, tr_w, use_w, ts, gs, a);
+        }
+      }
+      if constexpr (loss) {
+        // ... and leave transposed, 2 frows bytes per expert: thread (e, part) 8 rows of expert e
+        __syncthreads();
+        const int parts = frows / 8;
+        for (int i = threadIdx.x; i < N * parts; i += kWarpThreads) {
+          const int e = i / parts, r0 = i % parts * 8;
+          uint32_t w[4];
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const uint8_t* at = gsb + (r0 + 2 * r) * gpitch + e * 2;
+            w[r] = *reinterpret_cast<const uint16_t*>(at) |
+                   static_cast<uint32_t>(*reinterpret_cast<const uint16_t*>(at + gpitch)) << 16;
+          }
+          *reinterpret_cast<uint4*>(a.gt + static_cast<int64_t>(e) * a.Tpad + tc + f0 + r0) =
+              make_uint4(w[0], w[1], w[2], w[3]);
+        }
+      }
     }
     if constexpr (predict) {
-      int ties = 0;
-      if (good && tw < a.T) ties = finish_predict_rows<kRows>(rows, ts, lv, a, count, hist_s);
       if (lane == 0 && ties != 0 && a.near_tie != nullptr)
         atomicAdd(reinterpret_cast<unsigned long long*>(a.near_tie),
                   static_cast<unsigned long long>(ties));
@@ -848,34 +916,6 @@ __global__ void __launch_bounds__(by_warps ? kWarpThreads : kThreads, 1)
         __syncthreads();
         int32_t* hrow = a.hist + static_cast<int64_t>(blockIdx.x) * N;
         for (int e = threadIdx.x; e < N; e += kWarpThreads) hrow[e] = hist_s[e];
-      }
-    } else if constexpr (kMode == kModeReplay) {
-      if (tw < a.T) finish_replay_rows<kRows>(rows, es_w, ts, lv, a);
-    } else {
-      // the bf16 dKL/dz rows meet in shared memory and leave transposed, 2 kR bytes per expert
-      uint8_t* gsb = reinterpret_cast<uint8_t*>(rm + kR * pitch4);
-      const int gpitch = N * 2 + 8;
-      uint2* gs[kRows];
-#pragma unroll
-      for (int j = 0; j < kRows; ++j) {
-        gs[j] = reinterpret_cast<uint2*>(gsb + (wr0 + j) * gpitch + lane * 8);
-        use_w[j] = use_w[j] && good;
-      }
-      finish_loss_rows<kRows>(rows, po_w, tr_w, use_w, ts, gs, a);
-      __syncthreads();
-      // thread (e, part): 8 rows of expert e, one 16-byte store
-      constexpr int kParts = kR / 8;
-      for (int i = threadIdx.x; i < N * kParts; i += kWarpThreads) {
-        const int e = i / kParts, r0 = i % kParts * 8;
-        uint32_t w[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const uint8_t* at = gsb + (r0 + 2 * r) * gpitch + e * 2;
-          w[r] = *reinterpret_cast<const uint16_t*>(at) |
-                 static_cast<uint32_t>(*reinterpret_cast<const uint16_t*>(at + gpitch)) << 16;
-        }
-        *reinterpret_cast<uint4*>(a.gt + static_cast<int64_t>(e) * a.Tpad + t0 + rank * kR + r0) =
-            make_uint4(w[0], w[1], w[2], w[3]);
       }
     }
     tc_fence_before();
@@ -894,7 +934,7 @@ __global__ void __launch_bounds__(by_warps ? kWarpThreads : kThreads, 1)
     if (have) {
       float* lrow = (predict && a.logits_or_probs != nullptr && live) ? a.logits_or_probs + t * N
                                                                       : nullptr;
-      for (int c0 = fe0; c0 < fe0 + nr; c0 += 16) {
+      for (int c0 = 0; c0 < N; c0 += 16) {
         float z[16];
         if (predict) {
           uint32_t rp[16], rb[16];
@@ -938,24 +978,10 @@ __global__ void __launch_bounds__(by_warps ? kWarpThreads : kThreads, 1)
         }
       }
     }
-    // Combine the S threads of the row (consecutive lanes): max, rescaled sum, merged lists.
-    float mx = m;
-#pragma unroll
-    for (int o = 1; o < split; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    float fs = have ? sum * expf(m - mx) : 0.f;
-#pragma unroll
-    for (int o = 1; o < split; o <<= 1) fs += __shfl_xor_sync(0xffffffffu, fs, o);
-    const float inv_s = 1.0f / fs;
+    const float mx = m;
+    const float inv_s = 1.0f / sum;
     if (predict) {
-#pragma unroll
-      for (int o = 1; o < split; o <<= 1) {
-        uint64_t other[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j)
-          other[j] = j < kKeep ? __shfl_xor_sync(0xffffffffu, top[j], o) : 0ull;
-        merge16_desc(top, other);
-      }
-      if (have && live && part == 0) {
+      if (have && live) {
         tie = predict_write(top, mx, inv_s, t, a);
         if (count)
 #pragma unroll
@@ -963,12 +989,7 @@ __global__ void __launch_bounds__(by_warps ? kWarpThreads : kThreads, 1)
             if (j < k) atomicAdd(&hist_s[key_e(top[j])], 1);
       }
     } else if (!loss) {
-      // Each valid slot's z is held by the one thread owning its expert; the others hold 0.
-#pragma unroll
-      for (int s = 0; s < kMaxTopK; ++s)
-#pragma unroll
-        for (int o = 1; o < split; o <<= 1) z_s[s] += __shfl_xor_sync(0xffffffffu, z_s[s], o);
-      if (have && live && part == 0) {
+      if (have && live) {
         float* grow = a.gates + t * k;
         float gv[kMaxTopK];
         float sk = 0.f;
@@ -985,7 +1006,7 @@ __global__ void __launch_bounds__(by_warps ? kWarpThreads : kThreads, 1)
       }
       if (have && a.logits_or_probs != nullptr) {
         float* prow = a.logits_or_probs + t * N;
-        for (int c0 = fe0; c0 < fe0 + nr; c0 += 16) {
+        for (int c0 = 0; c0 < N; c0 += 16) {
           uint32_t rp[16];
           load16(c0, rp);
           if (live) {
@@ -1011,157 +1032,6 @@ __global__ void __launch_bounds__(by_warps ? kWarpThreads : kThreads, 1)
     }
     tc_fence_before();
   }
-  if (epi && loss && !by_warps) {
-    // Predictive loss (Eq. pr2_loss, Algorithm 3) of cached row t over experts [fe0, fe0+nr):
-    //   standard: prediction Softmax(v), v = p_old + b;  target rho (row pos[t] of the teacher)
-    //   delta:    prediction Softmax(b);  target Softmax(u), u = log rho - p_old
-    // KL_t = sum_j tgt_j (log tgt_j - log pred_j);  dKL_t/dv_j = pred_j - tgt_j, stored bf16
-    // and transposed for the gradient GEMM.  Two passes: normalisers, then terms.  The first
-    // kLossPre experts come from registers, any further ones from global memory.  Exponentials
-    // and logarithms use the hardware approximations (__expf, __logf: a few ulp over the ranges
-    // met here, far inside the loss's tolerance), which cut this phase from ~10 to ~4 us.
-    const bool delta = a.delta != 0;
-    if (live && !okp && part == 0 && a.status != nullptr) atomicOr(a.status, PR2_STATUS_BAD_INDEX);
-    const bool use = have && okp;
-    const float* po = a.p_old + (live ? t : 0) * N;
-    const float* tr = a.rho + (okp ? lrow : 0) * N;
-    auto row16 = [&](const float* src, int c, float (&v)[16]) {
-      const float4* q = reinterpret_cast<const float4*>(src + c);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float4 x = q[j];
-        v[4 * j] = x.x;
-        v[4 * j + 1] = x.y;
-        v[4 * j + 2] = x.z;
-        v[4 * j + 3] = x.w;
-      }
-    };
-    float m1 = -FLT_MAX, s1 = 0.f, m2 = -FLT_MAX, s2 = 0.f;
-    auto normalisers = [&](const uint32_t (&rb)[16], const float (&pv)[16],
-                           const float (&rv)[16]) {
-      float v[16], u[16];
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const float b = __uint_as_float(rb[j]);
-        v[j] = delta ? b : pv[j] + b;
-        u[j] = rv[j] > 0.f ? __logf(rv[j]) - pv[j] : -INFINITY;
-      }
-      float cm = v[0];
-#pragma unroll
-      for (int j = 1; j < 16; ++j) cm = fmaxf(cm, v[j]);
-      float nm = fmaxf(m1, cm), cs = 0.f;
-#pragma unroll
-      for (int j = 0; j < 16; ++j) cs += __expf(v[j] - nm);
-      s1 = s1 * __expf(m1 - nm) + cs;
-      m1 = nm;
-      if (delta) {
-        cm = u[0];
-#pragma unroll
-        for (int j = 1; j < 16; ++j) cm = fmaxf(cm, u[j]);
-        nm = fmaxf(m2, cm);
-        cs = 0.f;
-#pragma unroll
-        for (int j = 0; j < 16; ++j) cs += __expf(u[j] - nm);
-        s2 = s2 * __expf(m2 - nm) + cs;
-        m2 = nm;
-      }
-    };
-#pragma unroll
-    for (int ch = 0; ch < kLossPre / 16; ++ch) {
-      if (ch * 16 < nr) {
-        uint32_t rb[16];
-        load16(fe0 + ch * 16, rb);
-        if (use) {
-          float pv[16], rv[16];
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            pv[j] = po_s[ch * 16 + j];
-            rv[j] = tr_s[ch * 16 + j];
-          }
-          normalisers(rb, pv, rv);
-        }
-      }
-    }
-    for (int c0 = fe0 + kLossPre; c0 < fe0 + nr; c0 += 16) {
-      uint32_t rb[16];
-      load16(c0, rb);
-      if (use) {
-        float pv[16], rv[16];
-        row16(po, c0, pv);
-        row16(tr, c0, rv);
-        normalisers(rb, pv, rv);
-      }
-    }
-    float mx1 = m1, mx2 = m2;
-#pragma unroll
-    for (int o = 1; o < split; o <<= 1) {
-      mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, o));
-      mx2 = fmaxf(mx2, __shfl_xor_sync(0xffffffffu, mx2, o));
-    }
-    float f1 = s1 * __expf(m1 - mx1), f2 = s2 * __expf(m2 - mx2);
-#pragma unroll
-    for (int o = 1; o < split; o <<= 1) {
-      f1 += __shfl_xor_sync(0xffffffffu, f1, o);
-      f2 += __shfl_xor_sync(0xffffffffu, f2, o);
-    }
-    const float l1 = mx1 + __logf(f1), l2 = mx2 + __logf(f2);  // log normalisers
-    float kl = 0.f;
-    auto terms = [&](int c0, const uint32_t (&rb)[16], const float (&pv)[16],
-                     const float (&rv)[16]) {
-      float g[16];
-#pragma unroll
-      for (int j = 0; j < 16; ++j) g[j] = 0.f;
-      if (use) {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const float b = __uint_as_float(rb[j]);
-          const float lp = (delta ? b : pv[j] + b) - l1;  // log prediction
-          float tg, lt;
-          if (delta) {
-            lt = rv[j] > 0.f ? __logf(rv[j]) - pv[j] - l2 : -INFINITY;
-            tg = rv[j] > 0.f ? __expf(lt) : 0.f;
-          } else {
-            tg = rv[j];
-            lt = rv[j] > 0.f ? __logf(rv[j]) : 0.f;
-          }
-          if (tg > 0.f) kl += tg * (lt - lp);
-          g[j] = __expf(lp) - tg;
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 16; ++j)
-        a.gt[static_cast<int64_t>(c0 + j) * a.Tpad + t] =
-            __bfloat16_as_ushort(__float2bfloat16_rn(g[j]));
-    };
-#pragma unroll
-    for (int ch = 0; ch < kLossPre / 16; ++ch) {
-      if (ch * 16 < nr) {
-        uint32_t rb[16];
-        load16(fe0 + ch * 16, rb);
-        float pv[16], rv[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          pv[j] = use ? po_s[ch * 16 + j] : 0.f;
-          rv[j] = use ? tr_s[ch * 16 + j] : 0.f;
-        }
-        terms(fe0 + ch * 16, rb, pv, rv);
-      }
-    }
-    for (int c0 = fe0 + kLossPre; c0 < fe0 + nr; c0 += 16) {
-      uint32_t rb[16];
-      load16(c0, rb);
-      float pv[16], rv[16];
-      if (use) {
-        row16(po, c0, pv);
-        row16(tr, c0, rv);
-      }
-      terms(c0, rb, pv, rv);
-    }
-#pragma unroll
-    for (int o = 1; o < split; o <<= 1) kl += __shfl_xor_sync(0xffffffffu, kl, o);
-    if (live && part == 0) a.kl_tok[t] = use ? kl : 0.f;
-    tc_fence_before();
-  }
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
@@ -1170,26 +1040,27 @@ __global__ void __launch_bounds__(by_warps ? kWarpThreads : kThreads, 1)
   if (a.late_wait) pdl_wait();
 }
 
-template <int kMode, int kSplit, bool kWarps>
+template <int kMode, int kSplit, int kE>
 cudaError_t set_smem_attr(int N) {
-  const cudaError_t err = cudaFuncSetAttribute(route_tc_kernel<kMode, kSplit, kWarps>,
+  const cudaError_t err = cudaFuncSetAttribute(route_tc_kernel<kMode, kSplit, kE>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               route_layout(N, kMode == kModePredict, false).total);
+                                               route_layout(N, kMode, kSplit, false).total);
   if (err != cudaSuccess) return err;
   // all of the SM's unified L1 / shared storage as shared memory, so that two compact CTAs fit
-  return cudaFuncSetAttribute(route_tc_kernel<kMode, kSplit, kWarps>,
+  return cudaFuncSetAttribute(route_tc_kernel<kMode, kSplit, kE>,
                               cudaFuncAttributePreferredSharedMemoryCarveout,
                               cudaSharedmemCarveoutMaxShared);
 }
 
-template <int kMode, int kSplit, bool kWarps>
+template <int kMode, int kSplit, int kE>
 cudaError_t launch_kernel(const CUtensorMap& tm_h, const CUtensorMap& tm_w,
                           const CUtensorMap& tm_wp, const RouteTcArgs& a, int tiles,
                           cudaStream_t st, int* max_clusters) {
-  cudaError_t err = set_smem_attr<kMode, kSplit, kWarps>(a.N);
+  if (kE > 0 && a.compact != 0) return cudaErrorInvalidValue;  // no room for the rows
+  cudaError_t err = set_smem_attr<kMode, kSplit, kE>(a.N);
   if (err != cudaSuccess) return err;
-  const size_t smem = route_layout(a.N, kMode == kModePredict, a.compact != 0).total;
-  const dim3 block(kWarps ? kWarpThreads : kThreads);
+  const size_t smem = route_layout(a.N, kMode, kSplit, a.compact != 0).total;
+  const dim3 block(kE > 0 ? kWarpThreads : kThreads);
   if (max_clusters != nullptr) {  // occupancy query only
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(tiles * kSplit);
@@ -1202,10 +1073,10 @@ cudaError_t launch_kernel(const CUtensorMap& tm_h, const CUtensorMap& tm_w,
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaOccupancyMaxActiveClusters(max_clusters, route_tc_kernel<kMode, kSplit, kWarps>,
+    return cudaOccupancyMaxActiveClusters(max_clusters, route_tc_kernel<kMode, kSplit, kE>,
                                           &cfg);
   }
-  return launch_pdl(route_tc_kernel<kMode, kSplit, kWarps>, dim3(tiles * kSplit), block, smem, st,
+  return launch_pdl(route_tc_kernel<kMode, kSplit, kE>, dim3(tiles * kSplit), block, smem, st,
                     kSplit, tm_h, tm_w, tm_wp, a);
 }
 
@@ -1213,12 +1084,14 @@ template <int kMode, int kSplit>
 cudaError_t launch_split(const CUtensorMap& tm_h, const CUtensorMap& tm_w,
                          const CUtensorMap& tm_wp, const RouteTcArgs& a, int tiles,
                          cudaStream_t st, int* max_clusters) {
-  if constexpr (kSplit >= 4) {
-    const RouteSmemLayout L = route_layout(a.N, kMode == kModePredict, false);
-    if (route_by_warps(a.N, kSplit) && route_warps_bytes(L, kSplit) <= L.bar_offset)
-      return launch_kernel<kMode, kSplit, true>(tm_h, tm_w, tm_wp, a, tiles, st, max_clusters);
-  }
-  return launch_kernel<kMode, kSplit, false>(tm_h, tm_w, tm_wp, a, tiles, st, max_clusters);
+  if constexpr (kSplit == 1 && kMode != kModeLoss)
+    if (a.compact != 0 || a.N <= 128)
+      return launch_kernel<kMode, 1, 0>(tm_h, tm_w, tm_wp, a, tiles, st, max_clusters);
+  if (a.N > 128)
+    return launch_kernel<kMode, kSplit, 8>(tm_h, tm_w, tm_wp, a, tiles, st, max_clusters);
+  if (a.N > 64)
+    return launch_kernel<kMode, kSplit, 4>(tm_h, tm_w, tm_wp, a, tiles, st, max_clusters);
+  return launch_kernel<kMode, kSplit, 2>(tm_h, tm_w, tm_wp, a, tiles, st, max_clusters);
 }
 
 template <int kMode>
@@ -1254,9 +1127,9 @@ cudaError_t launch_any(int mode, const CUtensorMap& tm_h, const CUtensorMap& tm_
 // one SM side by side (a per-CTA %smid / %globaltimer record of a T = 32768 launch).
 template <int kMode>
 int compact_blocks_per_sm(int N) {
-  if (set_smem_attr<kMode, 1, false>(N) != cudaSuccess) return 0;
+  if (set_smem_attr<kMode, 1, 0>(N) != cudaSuccess) return 0;
   cudaFuncAttributes fa{};
-  if (cudaFuncGetAttributes(&fa, route_tc_kernel<kMode, 1, false>) != cudaSuccess) return 0;
+  if (cudaFuncGetAttributes(&fa, route_tc_kernel<kMode, 1, 0>) != cudaSuccess) return 0;
   int dev = 0, smem_sm = 0, reserved = 0, regs_sm = 0, threads_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) !=
@@ -1268,7 +1141,7 @@ int compact_blocks_per_sm(int N) {
       cudaDeviceGetAttribute(&threads_sm, cudaDevAttrMaxThreadsPerMultiProcessor, dev) !=
           cudaSuccess)
     return 0;
-  const size_t smem = route_layout(N, kMode == kModePredict, true).total + fa.sharedSizeBytes +
+  const size_t smem = route_layout(N, kMode, 1, true).total + fa.sharedSizeBytes +
                       static_cast<size_t>(reserved);
   const int regs = ((fa.numRegs + 7) / 8) * 8 * kThreads;  // allocated per warp in 256s
   int n = static_cast<int>(static_cast<size_t>(smem_sm) / smem);
@@ -1276,7 +1149,7 @@ int compact_blocks_per_sm(int N) {
   if (threads_sm / kThreads < n) n = threads_sm / kThreads;
   // each CTA holds its accumulator columns for its whole life: more CTAs than fit in the SM's
   // 512 TMEM columns would only wait in tcgen05.alloc for a neighbour to leave
-  const int b_rows = route_layout(N, kMode == kModePredict, true).b_rows;
+  const int b_rows = route_layout(N, kMode, 1, true).b_rows;
   const int by_tmem = static_cast<int>(512u / tmem_cols_for(b_rows));
   if (by_tmem < n) n = by_tmem;
   return n;
@@ -1326,27 +1199,17 @@ int max_active_clusters(int mode, int split, int N, bool compact = false) {
 bool route_compact(int T, int N, int mode, int num_sms) {
   const int tiles = (T + kTileM - 1) / kTileM;
   if (tiles <= num_sms) return false;
-  const RouteSmemLayout L = route_layout(N, mode == kModePredict, true);
+  const RouteSmemLayout L = route_layout(N, mode, 1, true);
   if (L.stages * L.stage_bytes > kCompactBudget) return false;  // not even two stages fit
   if (2 * tmem_cols_for(L.b_rows) > 512) return false;           // two accumulators in TMEM
   return max_active_clusters(mode, 1, N, true) >= 2 * num_sms;
 }
 
+// The widest cluster whose CTAs are all resident at once and have at least one K block each.
 int route_split(int T, int N, int d, int mode, int num_sms) {
-  const RouteSmemLayout L = route_layout(N, mode == kModePredict, false);
   const int tiles = (T + kTileM - 1) / kTileM;
-  const int KB = d / kBK;
-  if (L.passes == 2) {
-    // predict with N > 128: the pass split (two CTAs per tile, each receiving its 64 rows' two
-    // column halves) when it fits in one wave, else one CTA per tile streaming both passes
-    const bool fits = route_recv_bytes(L.b_rows) / 2 <= L.stages * L.stage_bytes &&
-                      KB % 2 == 0 && (N / 2) % 16 == 0 && tiles * 2 <= num_sms &&
-                      max_active_clusters(mode, 2, N) >= tiles;
-    return fits ? 2 : 1;
-  }
-  if (route_recv_bytes(L.b_rows) > L.stages * L.stage_bytes) return 1;
   for (int s = kMaxSplit; s > 1; s >>= 1) {
-    if (N % s != 0 || (N / s) % 16 != 0 || KB % s != 0 || tiles * s > num_sms) continue;
+    if (d / kBK < s || tiles * s > num_sms) continue;
     if (max_active_clusters(mode, s, N) < tiles) continue;  // must fit in one wave
     return s;
   }
@@ -1357,8 +1220,7 @@ cudaError_t launch_route_tc(int mode, const CUtensorMap& tm_h, const CUtensorMap
                             const CUtensorMap& tm_wp, const RouteTcArgs& a, int split,
                             cudaStream_t st) {
   if (a.T == 0) return cudaSuccess;
-  if (split < 1 || split > kMaxSplit || a.N % split != 0 || (a.N / split) % 16 != 0 ||
-      (a.d / kBK) % split != 0 || (a.compact != 0 && split != 1))
+  if (split < 1 || split > kMaxSplit || a.d / kBK < split || (a.compact != 0 && split != 1))
     return cudaErrorInvalidValue;
   const int tiles = (a.T + kTileM - 1) / kTileM;
   return launch_any(mode, tm_h, tm_w, tm_wp, a, split, tiles, st, nullptr);

@@ -1,5 +1,5 @@
-"""GPU parity of the predictive loss where its rows are finished by warps (64 < N <= 128, clusters
-of 4 and 8 CTAs): batches that end inside a CTA's rows, both objectives, teacher rows with zero
+"""GPU parity of the predictive loss where its rows are finished by warps (N = 128, clusters of 4
+and 8 CTAs): batches that end inside a CTA's rows, both objectives, teacher rows with zero
 entries and invalid cache positions.  Bounds as in the predictive-loss parity tests."""
 import numpy as np
 import pytest

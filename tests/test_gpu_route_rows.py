@@ -1,5 +1,5 @@
-"""GPU parity of predict routing where its rows are finished by warps (64 < N <= 128 in clusters of
-4 and 8 CTAs): batches that end inside a CTA's rows, in its first and last row and in a tile of few
+"""GPU parity of predict routing where its rows are finished by warps (N = 128 in clusters of 4 and
+8 CTAs): batches that end inside a CTA's rows, in its first and last row and in a tile of few
 rows (whose dead rows are not exchanged), every k, ties within and across the lanes' four experts
 (duplicated router rows: the lower expert first), with and without the logits and the
 renormalisation.  Routes, gates and logits against the oracle, tolerances of ``layer_harness``."""
