@@ -13,7 +13,7 @@
 //
 // What bounds it: the FMA issue rate for large layers, and the chain of K blocks at small ones;
 // hence two tile sizes (launch_expert_simt).  A rollout + replay step of the T = 256, d = 128,
-// m = 256, N = 8, k = 2 layer takes 79 us with these kernels and took 5203 us with one thread
+// m = 256, N = 8, k = 2 layer took 79 us when only these kernels had changed and 5203 us with one thread
 // per output column walking its weight row by uncoalesced 4-byte loads for every row of the
 // tile, behind a launch that wrote a permuted copy of h.
 #include "pr2_device.cuh"
@@ -207,11 +207,16 @@ cudaError_t launch_tile(bool swiglu, const SimtArgs& g, cudaStream_t st) {
 cudaError_t launch_expert_simt(bool swiglu, const SimtArgs& g, int64_t rows, int num_sms,
                                cudaStream_t st) {
   if (g.max_tiles <= 0) return cudaSuccess;
-  // 64 x 64 blocks move half the bytes per FMA of 32 x 32 ones, but only once they fill the GPU
-  // twice over; below that the shorter blocks win by their number.
-  const int64_t big = ((rows + 63) / 64) * ((g.n_out + 63) / 64);
-  return big >= 2 * static_cast<int64_t>(num_sms)
-             ? launch_tile<64, 64, 4, 4, 16>(swiglu, g, st)
+  // 32 x 64 blocks (4 x 4 per thread) read a third fewer bytes of shared memory per FMA than
+  // 32 x 32 ones (4 x 2), but only once they fill the GPU five times over; below that the shorter
+  // chains win by their number.  A rollout + replay step, 32 x 32 / 32 x 64 / 64 x 64: T = 2048,
+  // d = m = 512, N = 64, k = 8 1609 / 1473 / 1641 us; T = 600, m = 300 460 / 436 / 509; T = 2048,
+  // d = m = 256, N = 32, k = 4 262 / 256 / 290; T = 300, d = m = 400, N = 40, k = 4 202 / 260 / 239.
+  // Larger register tiles (8 x 4, 8 x 8) and packed FMAs (fma.rn.f32x2, even and odd K apart) gave
+  // nothing: 1556 and 1541 at the first of these sizes, the FMA pipe at 55 to 60 % either way.
+  const int64_t wide = ((rows + 31) / 32) * ((g.n_out + 63) / 64);
+  return wide >= 5 * static_cast<int64_t>(num_sms)
+             ? launch_tile<32, 64, 4, 4, 16>(swiglu, g, st)
              : launch_tile<32, 32, 4, 2, 32>(swiglu, g, st);
 }
 

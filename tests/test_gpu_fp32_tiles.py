@@ -1,5 +1,5 @@
-"""GPU parity of the fp32 grouped GEMM at the edges of its blocks: both block sizes (64 x 64
-once they fill the GPU twice), K blocks with a remainder, an expert width that is no multiple of 4
+"""GPU parity of the fp32 grouped GEMM at the edges of its blocks: both block sizes (32 x 64
+once they fill the GPU five times), K blocks with a remainder, an expert width that is no multiple of 4
 (unaligned rows, copied 4 bytes at a time), a last column block of one column, shared experts and
 experts without any row.  Compared in full with the oracle, tolerances of ``layer_harness``."""
 import pytest
@@ -16,7 +16,7 @@ CASES = {
     "one_column_over": dict(T=129, d=132, N=64, k=1, m=65, n_shared=1),
     "empty_experts": dict(T=3, d=4, N=200, k=2, m=31),
     "large_blocks": dict(T=2051, d=196, N=12, k=8, m=260, n_shared=2),
-    "large_blocks_ragged": dict(T=2500, d=256, N=3, k=3, m=129),
+    "large_blocks_ragged": dict(T=2700, d=256, N=3, k=3, m=129),
 }
 
 
