@@ -22,7 +22,8 @@ SHAPES = [(1, 16, 512, 4), (77, 80, 576, 8), (300, 144, 704, 8), (513, 256, 2112
           (900, 208, 320, 3), (2433, 240, 576, 8), (3001, 48, 832, 6), (4700, 256, 320, 8),
           (5003, 256, 192, 8), (5121, 176, 320, 5), (8200, 128, 448, 8), (9700, 64, 128, 8),
           (130, 64, 64, 2), (2000, 64, 1024, 6), (9800, 256, 128, 8), (10003, 224, 64, 8),
-          (9999, 128, 192, 8), (12001, 32, 64, 4), (19500, 256, 64, 8)]
+          (9999, 128, 192, 8), (12001, 32, 64, 4), (19500, 256, 64, 8),
+          (1100, 128, 2048, 8)]
 
 
 @pytest.mark.parametrize("T,N,d,k", SHAPES)
