@@ -24,13 +24,6 @@ namespace {
 
 constexpr int kStages = 3;
 
-// 4-byte asynchronous copy; src_bytes = 0 fills the word with zeros.
-__device__ __forceinline__ void cp_async_4(uint32_t smem_dst, const void* src, uint32_t src_bytes) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_dst), "l"(src),
-               "r"(src_bytes)
-               : "memory");
-}
-
 template <int BM, int BN, int TM, int TN, int BK, bool kSwiglu>
 struct SimtTile {
   static constexpr int kThreads = (BM / TM) * (BN / TN);

@@ -164,6 +164,12 @@ __device__ __forceinline__ void cp_async_16(uint32_t smem_dst, const void* src,
                "r"(src_bytes)
                : "memory");
 }
+// 4-byte asynchronous copy; src_bytes = 0 fills the word with zeros.
+__device__ __forceinline__ void cp_async_4(uint32_t smem_dst, const void* src, uint32_t src_bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_dst), "l"(src),
+               "r"(src_bytes)
+               : "memory");
+}
 // With an L2 eviction-priority hint (a createpolicy value).
 __device__ __forceinline__ void cp_async_16_hint(uint32_t smem_dst, const void* src,
                                                  uint32_t src_bytes, uint64_t policy) {
@@ -485,6 +491,27 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   uint32_t m;
   asm("mov.u32 %0, %lanemask_lt;" : "=r"(m));
   return m;
+}
+
+// Sum of each v[j] (j < 8) over the warp: returned in the lanes whose bits 4, 3, 2 are j.
+__device__ __forceinline__ float warp_sum8(const float (&v)[8]) {
+  const int lane = threadIdx.x & 31;
+  float a[4], b[2];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const bool hi = lane & 16;
+    a[j] = (hi ? v[j + 4] : v[j]) + __shfl_xor_sync(0xffffffffu, hi ? v[j] : v[j + 4], 16);
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const bool hi = lane & 8;
+    b[j] = (hi ? a[j + 2] : a[j]) + __shfl_xor_sync(0xffffffffu, hi ? a[j] : a[j + 2], 8);
+  }
+  const bool hi = lane & 4;
+  float c = (hi ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, hi ? b[0] : b[1], 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  c += __shfl_xor_sync(0xffffffffu, c, 1);
+  return c;
 }
 
 }  // namespace pr2

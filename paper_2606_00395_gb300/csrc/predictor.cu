@@ -10,7 +10,7 @@
 // chain is short); the cluster sums its fp32 partials, exchanged through L2, in split order and
 // scales by 1/T_c (deterministic), and the same launch sums the per-token KL in double in a fixed
 // order, so the loss call is two launches.
-// fp32: exact-fp32 SIMT kernels (one warp per cached token, one thread per gradient entry).
+// fp32: exact-fp32 SIMT kernels (warps over cached tokens, blocks over the gradient).
 #include <float.h>
 
 #include <mutex>
@@ -295,6 +295,7 @@ __global__ void __launch_bounds__(64)
 // ---- fp32 path ----------------------------------------------------------------------------
 
 constexpr int kPerLane = kMaxExperts / 32;
+constexpr int kLossWarps = 2;
 
 __device__ __forceinline__ float wsum(float v) {
 #pragma unroll
@@ -307,17 +308,14 @@ __device__ __forceinline__ float wmax(float v) {
   return v;
 }
 
-// One warp per cached token c; lane l holds experts e = 32 jj + l.
-__global__ void __launch_bounds__(256)
-    loss_simt_kernel(const float* __restrict__ h_old, const float* __restrict__ p_old,
-                     const float* __restrict__ Wp, const float* __restrict__ rho, int64_t T_rho,
-                     const int32_t* __restrict__ pos, int delta, int Tc, int d, int N,
-                     float* __restrict__ kl_tok, float* __restrict__ G, int32_t* status) {
-  pdl_wait();
-  pdl_trigger();
+// Loss terms of cached token c by one warp, from its predictor logits bz (lane l: experts 32 jj + l).
+__device__ __forceinline__ void loss_simt_row(int c, const float (&bz)[kPerLane],
+                                              const float* __restrict__ p_old,
+                                              const float* __restrict__ rho, int64_t T_rho,
+                                              const int32_t* __restrict__ pos, int delta, int N,
+                                              float* __restrict__ kl_tok, float* __restrict__ G,
+                                              int32_t* status) {
   const int lane = threadIdx.x & 31;
-  const int c = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (c >= Tc) return;
   const int64_t r = pos != nullptr ? static_cast<int64_t>(pos[c]) : c;
   float* grow = G + static_cast<int64_t>(c) * N;
   if (r < 0 || r >= T_rho) {
@@ -328,27 +326,18 @@ __global__ void __launch_bounds__(256)
     }
     return;
   }
-  const float* hc = h_old + static_cast<int64_t>(c) * d;
   float v[kPerLane], u[kPerLane], rv[kPerLane];
 #pragma unroll
   for (int jj = 0; jj < kPerLane; ++jj) {
-    v[jj] = -INFINITY;
-    u[jj] = -INFINITY;
+    const int e = jj * 32 + lane;
+    v[jj] = u[jj] = -INFINITY;
     rv[jj] = 0.f;
-    for (int l = 0; l < 32; ++l) {
-      const int e = jj * 32 + l;
-      if (e >= N) break;
-      const float* we = Wp + static_cast<int64_t>(e) * d;
-      float b = 0.f;
-      for (int i = lane; i < d; i += 32) b = fmaf(hc[i], we[i], b);
-      b = wsum(b);
-      if (lane == l) {
-        const float po = p_old[static_cast<int64_t>(c) * N + e];
-        const float tr = rho[r * N + e];
-        rv[jj] = tr;
-        v[jj] = delta ? b : po + b;
-        u[jj] = tr > 0.f ? logf(tr) - po : -INFINITY;
-      }
+    if (e < N) {
+      const float po = p_old[static_cast<int64_t>(c) * N + e];
+      const float tr = rho[r * N + e];
+      rv[jj] = tr;
+      v[jj] = delta ? bz[jj] : po + bz[jj];
+      u[jj] = tr > 0.f ? logf(tr) - po : -INFINITY;
     }
   }
   float m1 = -INFINITY, m2 = -INFINITY;
@@ -390,19 +379,135 @@ __global__ void __launch_bounds__(256)
   if (lane == 0) kl_tok[c] = kl;
 }
 
-// grad[j, i] = (1/T_c) sum_c G[c, j] h_old[c, i]; one thread per entry, consecutive i.
-__global__ void __launch_bounds__(256)
-    loss_grad_simt_kernel(const float* __restrict__ G, const float* __restrict__ h_old, int Tc,
-                          int d, int N, float* __restrict__ grad) {
+// One warp per kTok cached tokens; lane l holds experts e = 32 jj + l.  Eight experts at a time:
+// their predictor rows are read as float4 along d, all in flight, and the eight dot products summed
+// over the lanes together (as in the fp32 routing kernels, and for the same reasons).
+template <int kTok>
+__global__ void __launch_bounds__(kLossWarps * 32)
+    loss_simt_kernel(const float* __restrict__ h_old, const float* __restrict__ p_old,
+                     const float* __restrict__ Wp, const float* __restrict__ rho, int64_t T_rho,
+                     const int32_t* __restrict__ pos, int delta, int Tc, int d, int N,
+                     float* __restrict__ kl_tok, float* __restrict__ G, int32_t* status) {
   pdl_wait();
   pdl_trigger();
-  const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (idx >= static_cast<int64_t>(N) * d) return;
-  const int j = static_cast<int>(idx / d), i = static_cast<int>(idx % d);
-  float acc = 0.f;
-  for (int c = 0; c < Tc; ++c)
-    acc = fmaf(G[static_cast<int64_t>(c) * N + j], h_old[static_cast<int64_t>(c) * d + i], acc);
-  grad[idx] = Tc > 0 ? acc / static_cast<float>(Tc) : 0.f;
+  const int lane = threadIdx.x & 31;
+  const int c0 = (blockIdx.x * kLossWarps + (threadIdx.x >> 5)) * kTok;
+  if (c0 >= Tc) return;
+  const float* hc[kTok];
+#pragma unroll
+  for (int q = 0; q < kTok; ++q)
+    hc[q] = h_old + static_cast<int64_t>(c0 + q < Tc ? c0 + q : c0) * d;
+  float bz[kTok][kPerLane];  // predictor logits
+  const int src = ((lane & 4) << 2) | ((lane & 2) << 2) | ((lane & 1) << 2);
+#pragma unroll
+  for (int jj = 0; jj < kPerLane; ++jj) {
+#pragma unroll
+    for (int q = 0; q < kTok; ++q) bz[q][jj] = 0.f;
+    for (int g = 0; g < 4; ++g) {
+      const int e0 = jj * 32 + g * 8;
+      if (e0 >= N) break;
+      float b[kTok][8];
+#pragma unroll
+      for (int q = 0; q < kTok; ++q)
+#pragma unroll
+        for (int l = 0; l < 8; ++l) b[q][l] = 0.f;
+      for (int i = 4 * lane; i < d; i += 128) {
+        float4 x[kTok];
+#pragma unroll
+        for (int q = 0; q < kTok; ++q) x[q] = *reinterpret_cast<const float4*>(hc[q] + i);
+#pragma unroll
+        for (int l = 0; l < 8; ++l) {
+          const float4 w = __ldg(reinterpret_cast<const float4*>(
+              Wp + static_cast<int64_t>(e0 + l < N ? e0 + l : e0) * d + i));
+#pragma unroll
+          for (int q = 0; q < kTok; ++q)
+            b[q][l] = fmaf(x[q].w, w.w,
+                           fmaf(x[q].z, w.z, fmaf(x[q].y, w.y, fmaf(x[q].x, w.x, b[q][l]))));
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kTok; ++q) {
+        const float bs = __shfl_sync(0xffffffffu, warp_sum8(b[q]), src);
+        if ((lane >> 3) == g) bz[q][jj] = bs;
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < kTok; ++q)
+    if (c0 + q < Tc)
+      loss_simt_row(c0 + q, bz[q], p_old, rho, T_rho, pos, delta, N, kl_tok, G, status);
+}
+
+// grad[j, i] = (1/T_c) sum_c G[c, j] h_old[c, i], one chain of FMAs in ascending c per entry.  A
+// block of 128 threads owns 32 columns of h x 8 experts, 2 of them per thread; blocks of kGradTok
+// tokens travel through a ring of kGradStages stages as 4-byte cp.async copies (rows of G are not
+// 16-byte aligned for every N).  The chain over the tokens bounds it: with each entry's thread
+// loading its own operands the chain waited for L2 at every step.  Loss call before / with this
+// kernel and the row kernel above: T_c = 1024, d = 512, N = 64 223.8 / 77.2 us; T_c = 100, d = 500,
+// N = 50 98.5 / 26.4; T_c = 256, d = 256, N = 16 54.3 / 15.0.
+constexpr int kGradTok = 64;
+constexpr int kGradCols = 32, kGradRows = 8;
+constexpr int kGradStages = 3;
+__global__ void __launch_bounds__(128)
+    loss_grad_simt_kernel(const float* __restrict__ G, const float* __restrict__ h_old, int Tc,
+                          int d, int N, float* __restrict__ grad) {
+  __shared__ float hs[kGradStages][kGradTok][kGradCols];
+  __shared__ __align__(8) float gs[kGradStages][kGradTok][kGradRows];
+  const int col_blocks = (d + kGradCols - 1) / kGradCols;
+  const int i0 = static_cast<int>(blockIdx.x) % col_blocks * kGradCols;
+  const int j0 = static_cast<int>(blockIdx.x) / col_blocks * kGradRows;
+  const int tid = threadIdx.x, ti = tid & 31, tj = tid >> 5;
+  pdl_wait();
+  pdl_trigger();
+  auto issue = [&](int kb) {
+    const int st = kb % kGradStages, c0 = kb * kGradTok;
+#pragma unroll
+    for (int it = 0; it < kGradTok * kGradCols / 128; ++it) {
+      const int c = it * 4 + tj, i = i0 + ti;
+      const bool in = c0 + c < Tc && i < d;
+      cp_async_4(smem_u32(&hs[st][c][ti]), in ? h_old + static_cast<int64_t>(c0 + c) * d + i : h_old,
+                 in ? 4u : 0u);
+    }
+#pragma unroll
+    for (int it = 0; it < kGradTok * kGradRows / 128; ++it) {
+      const int c = it * 16 + (tid >> 3), j = j0 + (tid & 7);
+      const bool in = c0 + c < Tc && j < N;
+      cp_async_4(smem_u32(&gs[st][c][tid & 7]), in ? G + static_cast<int64_t>(c0 + c) * N + j : G,
+                 in ? 4u : 0u);
+    }
+  };
+  const int KB = (Tc + kGradTok - 1) / kGradTok;
+#pragma unroll
+  for (int s = 0; s < kGradStages - 1; ++s) {
+    if (s < KB) issue(s);
+    cp_async_commit();
+  }
+  float acc0 = 0.f, acc1 = 0.f;
+  for (int kb = 0; kb < KB; ++kb) {
+    cp_async_wait<kGradStages - 2>();
+    __syncthreads();  // stage kb has landed for every thread, stage kb - 1 is free
+    if (kb + kGradStages - 1 < KB) issue(kb + kGradStages - 1);
+    cp_async_commit();
+    const int st = kb % kGradStages;
+    const int n = Tc - kb * kGradTok < kGradTok ? Tc - kb * kGradTok : kGradTok;
+    auto step = [&](int c) {
+      const float2 g2 = *reinterpret_cast<const float2*>(&gs[st][c][2 * tj]);
+      const float x = hs[st][c][ti];
+      acc0 = fmaf(g2.x, x, acc0);
+      acc1 = fmaf(g2.y, x, acc1);
+    };
+    if (n == kGradTok) {
+#pragma unroll 16
+      for (int c = 0; c < kGradTok; ++c) step(c);
+    } else {
+      for (int c = 0; c < n; ++c) step(c);
+    }
+  }
+  const int i = i0 + ti, j = j0 + 2 * tj;
+  if (i >= d) return;
+  if (j < N) grad[static_cast<int64_t>(j) * d + i] = Tc > 0 ? acc0 / static_cast<float>(Tc) : 0.f;
+  if (j + 1 < N)
+    grad[static_cast<int64_t>(j + 1) * d + i] = Tc > 0 ? acc1 / static_cast<float>(Tc) : 0.f;
 }
 
 }  // namespace
@@ -514,15 +619,21 @@ cudaError_t launch_loss_simt(const float* h_old, const float* p_old, const float
                              int Tc, int d, int N, float* kl_tok, float* G, int32_t* status,
                              cudaStream_t st) {
   if (Tc == 0) return cudaSuccess;
-  return launch_pdl(loss_simt_kernel, dim3((Tc + 7) / 8), dim3(256), 0, st, 1, h_old, p_old, Wp,
-                    rho, T_rho, pos, delta, Tc, d, N, kl_tok, G, status);
+  // four tokens per warp where the predictor rows weigh more than the parallelism (as in routing)
+  const bool four = Tc >= 512 && static_cast<int64_t>(N) * d >= 16384;
+  const int per_block = kLossWarps * (four ? 4 : 1);
+  return launch_pdl(four ? loss_simt_kernel<4> : loss_simt_kernel<1>,
+                    dim3((Tc + per_block - 1) / per_block), dim3(kLossWarps * 32), 0, st, 1, h_old,
+                    p_old, Wp, rho, T_rho, pos, delta, Tc, d, N, kl_tok, G, status);
 }
 
 cudaError_t launch_loss_grad_simt(const float* G, const float* h_old, int Tc, int d, int N,
                                   float* grad, cudaStream_t st) {
-  const int64_t n = static_cast<int64_t>(N) * d;
-  return launch_pdl(loss_grad_simt_kernel, dim3(static_cast<unsigned>((n + 255) / 256)),
-                    dim3(256), 0, st, 1, G, h_old, Tc, d, N, grad);
+  const int64_t blocks = static_cast<int64_t>((d + kGradCols - 1) / kGradCols) *
+                         ((N + kGradRows - 1) / kGradRows);
+  if (blocks > INT32_MAX) return cudaErrorInvalidValue;
+  return launch_pdl(loss_grad_simt_kernel, dim3(static_cast<unsigned>(blocks)), dim3(128), 0, st,
+                    1, G, h_old, Tc, d, N, grad);
 }
 
 }  // namespace pr2

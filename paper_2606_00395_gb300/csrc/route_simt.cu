@@ -19,27 +19,6 @@ namespace {
 
 constexpr int kWarps = 2;
 
-// Sum of each v[j] (j < 8) over the warp: returned in the lanes whose bits 4, 3, 2 are j.
-__device__ __forceinline__ float warp_sum8(const float (&v)[8]) {
-  const int lane = threadIdx.x & 31;
-  float a[4], b[2];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const bool hi = lane & 16;
-    a[j] = (hi ? v[j + 4] : v[j]) + __shfl_xor_sync(0xffffffffu, hi ? v[j] : v[j + 4], 16);
-  }
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const bool hi = lane & 8;
-    b[j] = (hi ? a[j + 2] : a[j]) + __shfl_xor_sync(0xffffffffu, hi ? a[j] : a[j + 2], 8);
-  }
-  const bool hi = lane & 4;
-  float c = (hi ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, hi ? b[0] : b[1], 4);
-  c += __shfl_xor_sync(0xffffffffu, c, 2);
-  c += __shfl_xor_sync(0xffffffffu, c, 1);
-  return c;
-}
-
 template <bool kPredict, int kTok>
 __global__ void __launch_bounds__(kWarps * 32)
     route_simt_kernel(int T, int d, int N, int k, const float* __restrict__ h,
