@@ -669,11 +669,14 @@ cudaError_t launch_rows(const ExpertMaps& tm, const MlpArgs& a, int num_sms, cud
 }  // namespace
 
 // Tiles of 128 rows leave 48 KB more for the weight ring, tiles of 256 read an expert's weights and
-// issue its MMAs once for twice the rows.  Replay layer of the Qwen3 shape, 128 / 256 rows: 16
-// rows per expert 204 / 212 us, 64 219 / 226, 112 235 / 238, 128 251 / 243, 160 297 / 261; with
-// Zipf(1.2) routes 64 235 / 232, 96 261 / 253.
+// issue its MMAs once for twice the rows.  Replay layer of the Qwen3 shape, 128 / 256 rows, by mean
+// rows per expert: even routes 53 209.5 / 215.1 us, 69 213.4 / 218.7, 98 221.5 / 225.6, 119 231.5 /
+// 232.0, 131 249.1 / 235.9; Zipf(1.2) routes 32 207.7 / 212.6, 48 220 / 217.2, 64 230.6 / 223.3, 96
+// 259.8 / 245.5.  The line lies where the loss on either side is the same.  (One kernel that picks
+// the layout on the device by how many experts have more than 128 rows took 2 us more at every
+// size: more code to fetch after weights that flush L2.)
 int expert_tile_rows(int64_t rows, int N) {
-  return rows <= static_cast<int64_t>(N) * 96 ? 128 : 256;
+  return rows <= static_cast<int64_t>(N) * 64 ? 128 : 256;
 }
 
 cudaError_t launch_expert_tc(const ExpertMaps& tm, const MlpArgs& a, int tile_rows, int num_sms,
