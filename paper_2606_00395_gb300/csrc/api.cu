@@ -457,12 +457,12 @@ pr2_status moe_forward_impl(const pr2_dims* dims, const void* h, const int32_t* 
 
   const int64_t F = dm.T * dm.k;
   const int tile_rows = dm.dtype == PR2_BF16 ? expert_tile_rows(F, dm.N) : kMinTileRows;
-  // the caller's counts and perm, where given, are written (and perm read) in place of the
-  // workspace's
+  // The caller's counts, which no kernel reads, are written in place; perm, which the gate/up GEMM
+  // reads, is the workspace's and copied out at the end: callers may share one perm buffer
+  // between streams, as they may any output.
   int32_t* const counts_w = counts != nullptr ? counts : w.counts;
-  int32_t* const perm_w = perm != nullptr ? perm : w.perm;
   DispatchArgs da{idx,       dm.T,   dm.k,  dm.N,    dm.n_shared, w.blk_hist, counts_w,
-                  w.offsets, perm_w, w.inv, w.tiles, w.num_tiles, status,     w.sync_ctr,
+                  w.offsets, w.perm, w.inv, w.tiles, w.num_tiles, status,     w.sync_ctr,
                   dm.dtype == PR2_BF16 ? w.ready : nullptr, tile_rows};
   if (err == cudaSuccess)
     err = (rhist != nullptr && dm.dtype == PR2_BF16)
@@ -486,7 +486,7 @@ pr2_status moe_forward_impl(const pr2_dims* dims, const void* h, const int32_t* 
       tm.s_down = tm.down;
     }
     if (!ok) return PR2_ERR_CUDA;
-    const MlpArgs ma{w.tiles, w.num_tiles, w.max_tiles, w.ready, h,      perm_w, dm.k,
+    const MlpArgs ma{w.tiles, w.num_tiles, w.max_tiles, w.ready, h,      w.perm, dm.k,
                      dm.N,    dm.d,        dm.m,        w.hbuf,  w.ybuf, status};
     err = launch_expert_tc(tm, ma, tile_rows, num_sms, st);
     mark(events ? events->gate_up_done : nullptr);
@@ -495,11 +495,11 @@ pr2_status moe_forward_impl(const pr2_dims* dims, const void* h, const int32_t* 
     auto f32 = [](const void* p) { return static_cast<const float*>(p); };
     const int64_t rows = F + dm.n_shared * dm.T;
     SimtArgs g{w.tiles, w.num_tiles, w.max_tiles, dm.d, dm.m, dm.k, dm.N, f32(h), f32(W_gate),
-               f32(W_up), f32(Ws_gate), f32(Ws_up), perm_w, static_cast<float*>(w.hbuf), status};
+               f32(W_up), f32(Ws_gate), f32(Ws_up), w.perm, static_cast<float*>(w.hbuf), status};
     err = launch_expert_simt(true, g, rows, num_sms, st);
     mark(events ? events->gate_up_done : nullptr);
     SimtArgs g2{w.tiles, w.num_tiles, w.max_tiles, dm.m, dm.d, dm.k, dm.N, f32(w.hbuf),
-                f32(W_down), nullptr, f32(Ws_down), nullptr, perm_w, static_cast<float*>(w.ybuf),
+                f32(W_down), nullptr, f32(Ws_down), nullptr, w.perm, static_cast<float*>(w.ybuf),
                 status};
     if (err == cudaSuccess) err = launch_expert_simt(false, g2, rows, num_sms, st);
     mark(events ? events->down_done : nullptr);
@@ -521,6 +521,8 @@ pr2_status moe_forward_impl(const pr2_dims* dims, const void* h, const int32_t* 
                  dm.n_shared, dm.dtype == PR2_BF16 ? 1 : 0, out, residual, status};
   err = launch_combine(ca, num_sms, st);
   mark(events ? events->end : nullptr);
+  if (err == cudaSuccess && perm != nullptr)
+    err = cudaMemcpyAsync(perm, w.perm, sizeof(int32_t) * F, cudaMemcpyDeviceToDevice, st);
   return finish(err, dm.flags, status, st);
 }
 
