@@ -334,9 +334,11 @@ __global__ void __launch_bounds__(kSmallSlots)
   }
 }
 
-size_t small_smem_bytes(int N) {
+constexpr size_t small_smem_bytes(int N) {
   return sizeof(int) * (static_cast<size_t>(kSmallGroups) * N + 2 * N + 2);
 }
+// (with its static arrays) below the 48 KB that every kernel may take without an attribute
+static_assert(small_smem_bytes(kMaxExperts) + 5 * 1024 <= 48 * 1024, "dispatch_small_kernel");
 
 // Hist, scan and place in one cooperative launch (N % 4 == 0, N <= 256; grid resident): blocks of
 // kThr threads, kSlots slots per thread (f = base + c kThr + tid).  <256, 1> for most batches;
@@ -613,16 +615,21 @@ __global__ void __launch_bounds__(kHistBlock)
 
 constexpr int kFewBlocks = 384;
 
-size_t hist_smem_bytes(int N) { return sizeof(int) * (static_cast<size_t>(kHistWarps) * N + 4 * N + 2); }
+constexpr size_t hist_smem_bytes(int N) {
+  return sizeof(int) * (static_cast<size_t>(kHistWarps) * N + 4 * N + 2);
+}
+static_assert(hist_smem_bytes(kMaxExperts) + 1024 <= 48 * 1024, "dispatch_hist_kernel");
 
-size_t fused_smem_bytes(int N, int groups) {
+constexpr size_t fused_smem_bytes(int N, int groups) {
   return sizeof(int) * (static_cast<size_t>(groups) * N + 4 * N + 2);
 }
 
-cudaError_t set_large_fused_smem(int N) {
+// The limit is the kernel's, not the launch's: set to what the most experts need, so that a call
+// with fewer experts on another host thread cannot lower it between this and a launch.
+cudaError_t set_large_fused_smem() {
   return cudaFuncSetAttribute(dispatch_fused_kernel<1024, 2>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(fused_smem_bytes(N, 64)));
+                              static_cast<int>(fused_smem_bytes(kDispatchChunk, 64)));
 }
 
 // Blocks of the fused dispatch that fit on one SM (0 on error), cached per device, N and shape.
@@ -640,8 +647,7 @@ int fused_blocks_per_sm(int N, bool large) {
     if (cache[i].dev == dev && cache[i].N == N && cache[i].large == static_cast<int>(large))
       return cache[i].blocks_per_sm;
   int per_sm = 0;
-  const cudaError_t err =
-      large ? set_large_fused_smem(N) : cudaSuccess;
+  const cudaError_t err = large ? set_large_fused_smem() : cudaSuccess;
   if (err != cudaSuccess ||
       (large ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
                    &per_sm, dispatch_fused_kernel<1024, 2>, 1024, fused_smem_bytes(N, 64))
@@ -919,19 +925,15 @@ cudaError_t launch_dispatch(const DispatchArgs& a, int num_sms, cudaStream_t st)
   cudaError_t err = cudaSuccess;
   // One block for a small batch, any N (stage times with N = 128, k = 8: 128 slots 10.8 us by the
   // cooperative launch, 10.1 in one block; 512 11.9 / 10.5; 2048, two slots per thread 13.2 / 13.7)
-  if (F > 0 && F <= kSmallSlots) {
-    const size_t smem = small_smem_bytes(a.N);
-    err = cudaFuncSetAttribute(dispatch_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(smem));
-    if (err != cudaSuccess) return err;
-    return launch_pdl(dispatch_small_kernel, dim3(1), dim3(1024), smem, st, 1, a.idx,
+  if (F > 0 && F <= kSmallSlots && a.N <= kMaxExperts) {
+    return launch_pdl(dispatch_small_kernel, dim3(1), dim3(1024), small_smem_bytes(a.N), st, 1, a.idx,
                       static_cast<int>(F), a.k, a.N, a.T, a.n_shared, a.tile_rows, a.counts,
                       a.offsets, a.perm, a.inv, a.tiles, a.num_tiles, a.status, a.ready);
   }
   const int shape = a.sync_ctr != nullptr ? fused_dispatch_shape(a.N, F, num_sms) : 0;
   if (shape != 0) {
     err = cudaMemsetAsync(a.sync_ctr, 0, sizeof(unsigned int), st);
-    if (err == cudaSuccess && shape == 2) err = set_large_fused_smem(a.N);
+    if (err == cudaSuccess && shape == 2) err = set_large_fused_smem();
     if (err != cudaSuccess) return err;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(shape == 2 ? static_cast<unsigned>((F + 2047) / 2048) : nblk);
@@ -970,14 +972,10 @@ cudaError_t launch_dispatch_from_hist(const DispatchArgs& a, const int32_t* hist
                                       cudaStream_t st) {
   const int tiles_r = static_cast<int>((a.T + kTileM - 1) / kTileM);
   if (tiles_r == 0) return cudaSuccess;
-  if (a.N % 4 != 0 || a.k > kMaxTopK || hist == nullptr || split < 1) return cudaErrorInvalidValue;
-  const size_t smem = hist_smem_bytes(a.N);
-  cudaError_t err = cudaFuncSetAttribute(dispatch_hist_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-  if (err != cudaSuccess) return err;
-  return launch_pdl(dispatch_hist_kernel, dim3(tiles_r), dim3(kHistBlock), smem, st, 1, a.idx,
-                    a.T, a.k, a.N, a.n_shared, a.tile_rows, hist, tiles_r * split, split,
+  if (a.N % 4 != 0 || a.N > kMaxExperts || a.k > kMaxTopK || hist == nullptr || split < 1)
+    return cudaErrorInvalidValue;
+  return launch_pdl(dispatch_hist_kernel, dim3(tiles_r), dim3(kHistBlock), hist_smem_bytes(a.N), st, 1,
+                    a.idx, a.T, a.k, a.N, a.n_shared, a.tile_rows, hist, tiles_r * split, split,
                     a.counts, a.offsets, a.perm, a.inv, a.tiles, a.num_tiles, a.ready);
 }
 

@@ -68,6 +68,8 @@ constexpr int kMaxStages = 12;
 constexpr int kStageBudget = 192 * 1024;    // pipeline stages of a CTA alone on its SM
 constexpr int kCompactBudget = 96 * 1024;   // two CTAs per SM (more token tiles than SMs)
 constexpr int kFinishBudget = 224 * 1024;   // exchange and finishing of a CTA alone on its SM
+constexpr int kAlignSlack = 1024, kBarBytes = 256;
+constexpr int kMostSmem = kAlignSlack + kFinishBudget + kBarBytes;  // no launch takes more
 
 struct RouteSmemLayout {
   int stages;
@@ -109,7 +111,7 @@ __host__ __device__ inline RouteSmemLayout route_layout(int N, int mode, int spl
     const int need = L.xcols * kTileM * 4 + L.frows * row;
     if (need > L.bar_offset) L.bar_offset = (need + 15) & ~15;
   }
-  L.total = 1024 + L.bar_offset + 256;
+  L.total = kAlignSlack + L.bar_offset + kBarBytes;
   return L;
 }
 
@@ -1040,11 +1042,12 @@ __global__ void __launch_bounds__(kE > 0 ? kWarpThreads : kThreads, 1)
   if (a.late_wait) pdl_wait();
 }
 
+// The limit is the kernel's, not the launch's: the same for every shape, so that a call of another
+// shape on another host thread cannot lower it between this and a launch.
 template <int kMode, int kSplit, int kE>
-cudaError_t set_smem_attr(int N) {
-  const cudaError_t err = cudaFuncSetAttribute(route_tc_kernel<kMode, kSplit, kE>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               route_layout(N, kMode, kSplit, false).total);
+cudaError_t set_smem_attr() {
+  const cudaError_t err = cudaFuncSetAttribute(
+      route_tc_kernel<kMode, kSplit, kE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem);
   if (err != cudaSuccess) return err;
   // all of the SM's unified L1 / shared storage as shared memory, so that two compact CTAs fit
   return cudaFuncSetAttribute(route_tc_kernel<kMode, kSplit, kE>,
@@ -1057,9 +1060,10 @@ cudaError_t launch_kernel(const CUtensorMap& tm_h, const CUtensorMap& tm_w,
                           const CUtensorMap& tm_wp, const RouteTcArgs& a, int tiles,
                           cudaStream_t st, int* max_clusters) {
   if (kE > 0 && a.compact != 0) return cudaErrorInvalidValue;  // no room for the rows
-  cudaError_t err = set_smem_attr<kMode, kSplit, kE>(a.N);
+  cudaError_t err = set_smem_attr<kMode, kSplit, kE>();
   if (err != cudaSuccess) return err;
-  const size_t smem = route_layout(a.N, kMode, kSplit, a.compact != 0).total;
+  const int smem = route_layout(a.N, kMode, kSplit, a.compact != 0).total;
+  if (smem > kMostSmem) return cudaErrorInvalidValue;
   const dim3 block(kE > 0 ? kWarpThreads : kThreads);
   if (max_clusters != nullptr) {  // occupancy query only
     cudaLaunchConfig_t cfg = {};
@@ -1127,7 +1131,7 @@ cudaError_t launch_any(int mode, const CUtensorMap& tm_h, const CUtensorMap& tm_
 // one SM side by side (a per-CTA %smid / %globaltimer record of a T = 32768 launch).
 template <int kMode>
 int compact_blocks_per_sm(int N) {
-  if (set_smem_attr<kMode, 1, 0>(N) != cudaSuccess) return 0;
+  if (set_smem_attr<kMode, 1, 0>() != cudaSuccess) return 0;
   cudaFuncAttributes fa{};
   if (cudaFuncGetAttributes(&fa, route_tc_kernel<kMode, 1, 0>) != cudaSuccess) return 0;
   int dev = 0, smem_sm = 0, reserved = 0, regs_sm = 0, threads_sm = 0;
