@@ -66,3 +66,24 @@ def test_layers_from_two_threads(kind, T, k, dtype, Ns, n):
     assert [sum(c != 0 for c in side) for side in codes] == [0, 0]
     for (_, outs), ref in zip(sides, want):
         assert all(torch.equal(o, r) for o, r in zip(outs, ref))
+
+
+@pytest.mark.parametrize("kind", ["replay", "rollout"])
+def test_first_call_of_a_host_thread(kind):
+    """A thread whose first CUDA work is a routing call, on a stream that another thread made."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    B.load()
+    call, outs = _calls(kind, 40, 16, 4, "bf16")
+    B.check(call(None))
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    want = [o.clone() for o in outs]
+    torch.cuda.synchronize()
+    codes = []
+    thread = threading.Thread(target=lambda: codes.append(call(stream)))
+    thread.start()
+    thread.join()
+    stream.synchronize()
+    assert codes == [0]
+    assert all(torch.equal(o, w) for o, w in zip(outs, want))
