@@ -578,23 +578,25 @@ pr2_status rollout_impl(const pr2_dims* dims, const void* h, const void* W_route
   if (s != PR2_OK) return s;
   pr2_dims dr = dm;
   dr.flags &= ~PR2_F_SYNC_STATUS;
-  if (dm.dtype != PR2_BF16) {  // fp32: the two calls in sequence
-    s = route_common(&dr, true, h, W_router, W_pred, nullptr, idx, gates, logits_old, near_tie,
-                     status_dev, stream);
-    if (s != PR2_OK) return s;
-    return moe_forward_impl(dims, h, idx, gates, W_gate, W_up, W_down, Ws_gate, Ws_up, Ws_down,
-                            out, residual, counts, perm, workspace, ws_bytes, status_dev, events,
-                            stream);
-  }
   const Workspace w = carve(dm, static_cast<uint8_t*>(workspace));
+  // One status word for both steps, cleared before the first: a wait that runs out in the routing
+  // kernel keeps the kernels behind it from reading the route it did not write.
+  int32_t* status = status_dev;
+  if (status == nullptr) {
+    status = w.status;
+    if (cudaMemsetAsync(status, 0, sizeof(int32_t), static_cast<cudaStream_t>(stream)) != cudaSuccess)
+      return PR2_ERR_CUDA;
+  }
+  // bf16: the routing kernel leaves its per-CTA histograms for dispatch
+  const bool hist = dm.dtype == PR2_BF16;
   int split = 1;
   s = route_common(&dr, true, h, W_router, W_pred, nullptr, idx, gates, logits_old, near_tie,
-                   status_dev, stream, false, w.route_hist, &split);
+                   status, stream, false, hist ? w.route_hist : nullptr, &split);
   if (s != PR2_OK) return s;
   const RouteHist rh{w.route_hist, split};
   return moe_forward_impl(dims, h, idx, gates, W_gate, W_up, W_down, Ws_gate, Ws_up, Ws_down,
-                          out, residual, counts, perm, workspace, ws_bytes, status_dev, events,
-                          stream, nullptr, &rh);
+                          out, residual, counts, perm, workspace, ws_bytes, status, events,
+                          stream, nullptr, hist ? &rh : nullptr);
 }
 
 }  // namespace

@@ -500,7 +500,9 @@ __global__ void __launch_bounds__(kThr)
 // derives the expert totals and its own prefix from the histogram rows (int4 column reads),
 // then places its slots in stable order exactly as dispatch_fused_kernel does; block 0 writes
 // counts, offsets and the tile tables.  Every slot is valid (the routing kernel wrote k distinct
-// experts in [0, N) per token), which is what the histograms counted.
+// experts in [0, N) per token), which is what the histograms counted, unless a wait of the routing
+// kernel ran out: then its route may be unwritten, nothing is dispatched, and the GEMM and the
+// combine, which check the status word too, do nothing either.
 constexpr int kHistBlock = kTileM * kMaxTopK;  // 1024 threads: the slots of one routing tile
 constexpr int kHistWarps = kHistBlock / 32;
 
@@ -510,7 +512,7 @@ __global__ void __launch_bounds__(kHistBlock)
                          int split, int32_t* __restrict__ counts, int32_t* __restrict__ offsets,
                          int32_t* __restrict__ perm, int32_t* __restrict__ inv,
                          TileEntry* __restrict__ tiles, int32_t* __restrict__ num_tiles,
-                         int32_t* __restrict__ ready) {
+                         int32_t* __restrict__ ready, const int32_t* status) {
   extern __shared__ int dsm[];
   int* wcnt = dsm;                     // [kHistWarps][N] per-warp counts, then per-warp bases
   int* tot = wcnt + kHistWarps * N;    // [N]
@@ -527,6 +529,7 @@ __global__ void __launch_bounds__(kHistBlock)
   }
   pdl_wait();  // the route and its histograms come from the routing kernel
   pdl_trigger();
+  const bool dead = status_timed_out(status);  // acted on below, its load in flight until then
   __syncthreads();
   // ---- expert totals and this tile's prefix: hist rows [0, hist_rows), before = rows < b*split
   const int n4 = N / 4, G = kHistBlock / n4;
@@ -570,10 +573,11 @@ __global__ void __launch_bounds__(kHistBlock)
   const int64_t F = T * k;
   const int64_t f = static_cast<int64_t>(b) * kTileM * k + tid;
   const bool own = tid < kTileM * k && f < F;
-  const int e = own ? idx[f] : -1;
+  int e = own ? idx[f] : -1;
+  if (e < 0 || e >= N) e = -1;  // (an unwritten route: no index into shared memory)
   const unsigned same = __match_any_sync(0xffffffffu, e);
   if (e >= 0 && lane == __ffs(same) - 1) wcnt[w * N + e] = __popc(same);
-  __syncthreads();
+  if (__syncthreads_or(dead)) return;
   int all_rows, all_tiles;
   const int total = tid < N ? tot[tid] : 0;
   const int off = block_exclusive_scan<32>(total, sh, &all_rows);
@@ -607,9 +611,13 @@ __global__ void __launch_bounds__(kHistBlock)
   }
   __syncthreads();
   if (own) {
-    const int pos = wcnt[w * N + e] + __popc(same & lanemask_lt());
-    perm[pos] = static_cast<int32_t>(f);
-    inv[f] = pos;
+    if (e >= 0) {
+      const int pos = wcnt[w * N + e] + __popc(same & lanemask_lt());
+      perm[pos] = static_cast<int32_t>(f);
+      inv[f] = pos;
+    } else {
+      inv[f] = -1;
+    }
   }
 }
 
@@ -976,7 +984,7 @@ cudaError_t launch_dispatch_from_hist(const DispatchArgs& a, const int32_t* hist
     return cudaErrorInvalidValue;
   return launch_pdl(dispatch_hist_kernel, dim3(tiles_r), dim3(kHistBlock), hist_smem_bytes(a.N), st, 1,
                     a.idx, a.T, a.k, a.N, a.n_shared, a.tile_rows, hist, tiles_r * split, split,
-                    a.counts, a.offsets, a.perm, a.inv, a.tiles, a.num_tiles, a.ready);
+                    a.counts, a.offsets, a.perm, a.inv, a.tiles, a.num_tiles, a.ready, a.status);
 }
 
 cudaError_t launch_combine(const CombineArgs& a, int num_sms, cudaStream_t st) {
