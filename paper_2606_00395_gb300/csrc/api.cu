@@ -152,11 +152,14 @@ pr2_status finish(cudaError_t err, uint32_t flags, int32_t* status_dev, cudaStre
   return PR2_OK;
 }
 
+// `slice`: aux is a later layer's part of a buffer whose start has been checked.  In fp32 it starts
+// at any float (T N need not be a multiple of 4), where the fp32 kernels store single floats; in
+// bf16 N is a multiple of 16 and every part is aligned.
 pr2_status route_common(const pr2_dims* dims, bool predict, const void* h, const void* W,
                         const void* Wp, const int32_t* idx_in, int32_t* idx_out, float* gates,
                         float* aux, int64_t* near_tie, int32_t* status_dev, void* stream,
                         bool late_wait = false, int32_t* hist = nullptr,
-                        int* split_out = nullptr) {
+                        int* split_out = nullptr, bool slice = false) {
   pr2_status s = check_dims(dims);
   if (s != PR2_OK) return s;
   const pr2_dims& dm = *dims;
@@ -165,7 +168,7 @@ pr2_status route_common(const pr2_dims* dims, bool predict, const void* h, const
   if (predict && (Wp == nullptr || idx_out == nullptr)) return PR2_ERR_INVALID_ARG;
   if (!predict && idx_in == nullptr) return PR2_ERR_INVALID_ARG;
   if ((dm.flags & PR2_F_SYNC_STATUS) && status_dev == nullptr) return PR2_ERR_INVALID_ARG;
-  if (!aligned16(h) || !aligned16(W) || (Wp && !aligned16(Wp)) || (aux && !aligned16(aux)))
+  if (!aligned16(h) || !aligned16(W) || (Wp && !aligned16(Wp)) || (!slice && aux && !aligned16(aux)))
     return PR2_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t err;
@@ -556,14 +559,15 @@ pr2_status pr2_moe_forward(const pr2_dims* dims, const void* h, const int32_t* i
 namespace pr2 {
 namespace {
 
-// The rollout layer of pr2_moe_rollout_forward; `residual` as in moe_forward_impl.
+// The rollout layer of pr2_moe_rollout_forward; `residual` as in moe_forward_impl, `slice` (of
+// logits_old) as in route_common.
 pr2_status rollout_impl(const pr2_dims* dims, const void* h, const void* W_router,
                         const void* W_pred, int32_t* idx, float* gates, float* logits_old,
                         int64_t* near_tie, const void* W_gate, const void* W_up,
                         const void* W_down, const void* Ws_gate, const void* Ws_up,
                         const void* Ws_down, void* out, const void* residual, int32_t* counts,
                         int32_t* perm, void* workspace, size_t ws_bytes, int32_t* status_dev,
-                        const pr2_stage_events* events, void* stream) {
+                        const pr2_stage_events* events, void* stream, bool slice = false) {
   pr2_status s = check_dims(dims);
   if (s != PR2_OK) return s;
   const pr2_dims& dm = *dims;
@@ -571,7 +575,7 @@ pr2_status rollout_impl(const pr2_dims* dims, const void* h, const void* W_route
   if ((dm.flags & PR2_F_SYNC_STATUS) && status_dev == nullptr) return PR2_ERR_INVALID_ARG;
   // everything both steps need is checked before anything is launched
   if (W_router == nullptr || W_pred == nullptr || !aligned16(W_router) || !aligned16(W_pred) ||
-      (logits_old != nullptr && !aligned16(logits_old)))
+      (!slice && logits_old != nullptr && !aligned16(logits_old)))
     return PR2_ERR_INVALID_ARG;
   s = forward_args(dm, h, idx, gates, W_gate, W_up, W_down, Ws_gate, Ws_up, Ws_down, out,
                    workspace, ws_bytes);
@@ -591,7 +595,7 @@ pr2_status rollout_impl(const pr2_dims* dims, const void* h, const void* W_route
   const bool hist = dm.dtype == PR2_BF16;
   int split = 1;
   s = route_common(&dr, true, h, W_router, W_pred, nullptr, idx, gates, logits_old, near_tie,
-                   status, stream, false, hist ? w.route_hist : nullptr, &split);
+                   status, stream, false, hist ? w.route_hist : nullptr, &split, slice);
   if (s != PR2_OK) return s;
   const RouteHist rh{w.route_hist, split};
   return moe_forward_impl(dims, h, idx, gates, W_gate, W_up, W_down, Ws_gate, Ws_up, Ws_down,
@@ -671,7 +675,7 @@ pr2_status pr2_rollout_layers(const pr2_dims* dims, int32_t L, void* h, const vo
                      logits_l, near_tie, base(W_gate, l * gu_sz), base(W_up, l * gu_sz),
                      base(W_down, l * gu_sz), base(Ws_gate, l * sgu_sz), base(Ws_up, l * sgu_sz),
                      base(Ws_down, l * sgu_sz), h, h, nullptr, nullptr, workspace, ws_bytes,
-                     status_dev, nullptr, stream);
+                     status_dev, nullptr, stream, l > 0);
     if (s != PR2_OK) return s;
   }
   return finish(cudaSuccess, dm.flags, status_dev, static_cast<cudaStream_t>(stream));
