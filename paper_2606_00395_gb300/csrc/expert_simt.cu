@@ -75,7 +75,7 @@ __global__ void __launch_bounds__((SimtTile<BM, BN, TM, TN, BK, kSwiglu>::kThrea
     if (row < BM) {
       if (r0 + row < te.rows) {
         // gate/up: the token at this place (shared experts: the token itself); down: its H row
-        const int p = (kSwiglu ? te.a_row0 : te.out_row0) + r0 + row;
+        const uint32_t p = (kSwiglu ? static_cast<uint32_t>(te.a_row0) : te.out_row0) + r0 + row;
         src[i] = A + static_cast<int64_t>(kSwiglu && !shared ? g.perm[p] / g.k : p) * K + kc;
         on |= 1u << i;
       }

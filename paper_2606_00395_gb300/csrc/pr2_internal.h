@@ -39,7 +39,8 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 
 // One tile of a grouped GEMM: `rows` rows multiplied by the weights of `expert` (see MlpArgs).
 struct TileEntry {
-  int32_t expert, a_row0, rows, out_row0;
+  int32_t expert, a_row0, rows;
+  uint32_t out_row0;  // T k + n_shared T rows may pass 2^31 (fp32 layers of a few columns)
 };
 
 constexpr int kTileM = 128;         // tokens of a routing tile (one tcgen05 M=128 accumulator)
