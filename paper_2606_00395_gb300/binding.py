@@ -137,16 +137,14 @@ def _p(t: Optional[torch.Tensor]):
 
 _get_device = getattr(torch._C, "_cuda_getDevice", None)
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-_cuda_ready = False
 
 
 def _s(stream) -> int:
-    global _cuda_ready
     if stream is None:
-        if _cuda_ready:
+        # (not initialised: CUDA unused so far, or a process forked from one that used it)
+        if _raw_stream is not None and _get_device is not None and torch.cuda.is_initialized():
             return _raw_stream(_get_device())
         stream = torch.cuda.current_stream()  # initialises CUDA, or raises
-        _cuda_ready = _get_device is not None and _raw_stream is not None
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
