@@ -424,8 +424,10 @@ pr2_status forward_args(const pr2_dims& dm, const void* h, const int32_t* idx, c
     if (!aligned16(p)) return PR2_ERR_INVALID_ARG;
   if (dm.n_shared > 0 && (!aligned16(Ws_gate) || !aligned16(Ws_up) || !aligned16(Ws_down)))
     return PR2_ERR_INVALID_ARG;
-  // a tile's first row of H and Y is held in 32 bits (TileEntry)
-  if (dm.T * dm.k + dm.T * dm.n_shared > int64_t{UINT32_MAX}) return PR2_ERR_UNSUPPORTED;
+  // A tile's first row of H and Y is held in 32 bits (TileEntry), read as signed by the bf16 kernel:
+  // 2^31 rows of at least 64 columns would be 550 GB of H and Y.
+  const int64_t most = dm.dtype == PR2_BF16 ? int64_t{INT32_MAX} : int64_t{UINT32_MAX};
+  if (dm.T * dm.k + dm.T * dm.n_shared > most) return PR2_ERR_UNSUPPORTED;
   const Workspace probe = carve(dm, nullptr);
   if (workspace == nullptr || ws_bytes < probe.total ||
       (reinterpret_cast<uintptr_t>(workspace) & 255u) != 0)

@@ -123,11 +123,12 @@ __device__ void write_tile_table(int N, int64_t T, int k, int n_shared, int tile
       const int sz = ((c + nch - 1) / nch + 15) & ~15;  // (nch - 1) sz < c: no tile is empty
       const int r0 = ex_off[lo] + j * sz;
       const int left = ex_off[lo + 1] - r0;
-      tiles[i] = TileEntry{lo, r0, left < sz ? left : sz, static_cast<uint32_t>(r0)};
+      tiles[i] = TileEntry{lo, r0, left < sz ? left : sz, r0};
     } else {
       const int j = (i - routed) / per_shared, t0 = (i - routed) % per_shared * tile_rows;
       const int rows = T - t0 < tile_rows ? static_cast<int>(T - t0) : tile_rows;
-      tiles[i] = TileEntry{N + j, t0, rows, static_cast<uint32_t>(T * k + j * T + t0)};
+      const uint32_t out0 = static_cast<uint32_t>(T * k + j * T + t0);
+      tiles[i] = TileEntry{N + j, t0, rows, static_cast<int32_t>(out0)};
     }
   }
 }

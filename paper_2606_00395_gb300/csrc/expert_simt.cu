@@ -75,7 +75,7 @@ __global__ void __launch_bounds__((SimtTile<BM, BN, TM, TN, BK, kSwiglu>::kThrea
     if (row < BM) {
       if (r0 + row < te.rows) {
         // gate/up: the token at this place (shared experts: the token itself); down: its H row
-        const uint32_t p = (kSwiglu ? static_cast<uint32_t>(te.a_row0) : te.out_row0) + r0 + row;
+        const uint32_t p = static_cast<uint32_t>(kSwiglu ? te.a_row0 : te.out_row0) + r0 + row;
         src[i] = A + static_cast<int64_t>(kSwiglu && !shared ? g.perm[p] / g.k : p) * K + kc;
         on |= 1u << i;
       }
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__((SimtTile<BM, BN, TM, TN, BK, kSwiglu>::kThrea
   for (int i = 0; i < TM; ++i) {
     const int r = r0 + ty + kTy * i;
     if (r >= te.rows) continue;
-    float* orow = g.out + static_cast<int64_t>(te.out_row0 + r) * n_out;
+    float* orow = g.out + static_cast<int64_t>(static_cast<uint32_t>(te.out_row0) + r) * n_out;
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
       const int c = c0 + tx + kTx * j;

@@ -40,7 +40,10 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // One tile of a grouped GEMM: `rows` rows multiplied by the weights of `expert` (see MlpArgs).
 struct TileEntry {
   int32_t expert, a_row0, rows;
-  uint32_t out_row0;  // T k + n_shared T rows may pass 2^31 (fp32 layers of a few columns)
+  // 32 unsigned bits: T k + n_shared T rows may pass 2^31 in fp32 layers of a few columns.  Never in
+  // bf16 (refused by the host), whose kernel reads it as it is: with an unsigned field its code came
+  // out slower (Qwen3-shaped replay of 3001 tokens 257.3 -> 260.1 us, of 32768 1873 -> 1898).
+  int32_t out_row0;
 };
 
 constexpr int kTileM = 128;         // tokens of a routing tile (one tcgen05 M=128 accumulator)
