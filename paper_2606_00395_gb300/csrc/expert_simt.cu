@@ -61,6 +61,11 @@ __global__ void __launch_bounds__((SimtTile<BM, BN, TM, TN, BK, kSwiglu>::kThrea
   const int r0 = (row_block % kSub) * BM;
   if (r0 >= te.rows) return;
   const int c0 = (static_cast<int>(blockIdx.x) % col_blocks) * BN;
+  // the tile's first row: of A where rows are not gathered (gate/up of a shared expert: the token;
+  // down: the H row), and of the output
+  const int64_t row0 = static_cast<uint32_t>(te.out_row0);
+  const float* A0 = kSwiglu ? (shared ? A + static_cast<int64_t>(te.a_row0) * K : A) : A + row0 * K;
+  float* out0 = g.out + row0 * n_out;
   const int tid = threadIdx.x;
   const bool vec = K % 4 == 0;  // rows of 16-byte words (every base is 16-byte aligned)
 
@@ -74,9 +79,8 @@ __global__ void __launch_bounds__((SimtTile<BM, BN, TM, TN, BK, kSwiglu>::kThrea
     src[i] = A;
     if (row < BM) {
       if (r0 + row < te.rows) {
-        // gate/up: the token at this place (shared experts: the token itself); down: its H row
-        const uint32_t p = static_cast<uint32_t>(kSwiglu ? te.a_row0 : te.out_row0) + r0 + row;
-        src[i] = A + static_cast<int64_t>(kSwiglu && !shared ? g.perm[p] / g.k : p) * K + kc;
+        const int p = r0 + row;
+        src[i] = A0 + static_cast<int64_t>(kSwiglu && !shared ? g.perm[te.a_row0 + p] / g.k : p) * K + kc;
         on |= 1u << i;
       }
     } else {
@@ -171,7 +175,7 @@ __global__ void __launch_bounds__((SimtTile<BM, BN, TM, TN, BK, kSwiglu>::kThrea
   for (int i = 0; i < TM; ++i) {
     const int r = r0 + ty + kTy * i;
     if (r >= te.rows) continue;
-    float* orow = g.out + static_cast<int64_t>(static_cast<uint32_t>(te.out_row0) + r) * n_out;
+    float* orow = out0 + static_cast<int64_t>(r) * n_out;
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
       const int c = c0 + tx + kTx * j;
