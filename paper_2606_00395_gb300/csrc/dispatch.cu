@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(kHistBlock)
   }
   pdl_wait();  // the route and its histograms come from the routing kernel
   pdl_trigger();
-  const bool dead = status_timed_out(status);  // acted on below, its load in flight until then
+  const bool dead = tid == 0 && status_timed_out(status);  // acted on below, in flight until then
   __syncthreads();
   // ---- expert totals and this tile's prefix: hist rows [0, hist_rows), before = rows < b*split
   const int n4 = N / 4, G = kHistBlock / n4;
