@@ -1,8 +1,9 @@
-"""GPU parity of dispatch in each of its launch shapes: one block (up to 2048 slots, any number of
-experts), 256-slot blocks and 2048-slot blocks in one cooperative launch, at the edges between them
-and of their last block, with invalid and repeated route entries.  Counts and permutation are bit
-equal to the oracle's, the status word reports the invalid slots, and the layer output (which reads
-the tile table) matches."""
+"""GPU parity of dispatch in each of its launch shapes: one block (up to 1024 slots, any number of
+experts), 256-slot blocks (up to 98304 slots) and 2048-slot blocks in one cooperative launch, and
+three launches (numbers of experts that are no multiple of 4), at the edges between them and of
+their last block, with invalid and repeated route entries.  Counts and permutation are bit equal to
+the oracle's, the status word reports the invalid slots, and the layer output (which reads the tile
+table) matches."""
 import numpy as np
 import pytest
 import torch
@@ -21,11 +22,27 @@ pytestmark = pytest.mark.gpu
     (131073, 1, 16, True), (16385, 8, 32, False), (40000, 4, 64, True)])
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 def test_dispatch_shapes(T, k, N, bad, dtype):
+    _check(T, k, N + 4 if dtype == "fp32" and T > 2048 else N, bad, dtype)
+
+
+@pytest.mark.parametrize("T,k,N,bad,dtype", [
+    # 1023, 1024 and 1025 slots: the last of one block, the first of several
+    (341, 3, 16, True, "bf16"), (341, 3, 144, False, "bf16"), (341, 3, 256, True, "bf16"),
+    (128, 8, 16, False, "bf16"), (128, 8, 144, True, "bf16"), (256, 4, 256, True, "bf16"),
+    (205, 5, 16, True, "bf16"), (205, 5, 144, True, "bf16"), (205, 5, 256, False, "bf16"),
+    (341, 3, 5, True, "fp32"), (128, 8, 251, True, "fp32"), (205, 5, 131, True, "fp32"),
+    (64, 16, 33, True, "fp32"),
+    # 98304 and 98305 slots: the last in blocks of 256, the first in blocks of 2048
+    (12288, 8, 16, True, "bf16"), (24576, 4, 256, False, "bf16"),
+    (19661, 5, 16, False, "bf16"), (19661, 5, 256, True, "bf16"), (98305, 1, 6, True, "fp32")])
+def test_dispatch_edges(T, k, N, bad, dtype):
+    _check(T, k, N, bad, dtype)
+
+
+def _check(T, k, N, bad, dtype):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     B.load()
-    if dtype == "fp32" and T > 2048:
-        N += 4
     d, m = 64, 64
     cfg = synth.LayerConfig("d", T=T, d=d, N=N, k=k, m=m, dtype=dtype)
     L = synth.make_layer(cfg, seed=2)
