@@ -110,7 +110,7 @@ Workspace carve(const pr2_dims& dm, uint8_t* base) {
   const size_t es = esize(dm);
   w.nblk = static_cast<int>((F + kDispatchChunk - 1) / kDispatchChunk);
   const int mt_T = static_cast<int>((dm.T + kTileM - 1) / kTileM);
-  // tiles of at most 128 rows or more
+  // as many tiles as tiles of at most 128 rows are (those of at most 256 are fewer)
   w.max_tiles = static_cast<int>(F / kMinTileRows + dm.N + 1) +
                 dm.n_shared * static_cast<int>((dm.T + kMinTileRows - 1) / kMinTileRows);
   w.status = reinterpret_cast<int32_t*>(take(sizeof(int32_t)));
@@ -123,8 +123,8 @@ Workspace carve(const pr2_dims& dm, uint8_t* base) {
   w.sync_ctr = reinterpret_cast<unsigned int*>(take(sizeof(unsigned int)));
   w.ready = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * w.max_tiles));
   w.tiles = reinterpret_cast<TileEntry*>(take(sizeof(TileEntry) * w.max_tiles));
-  // fp32: the size that callers plan with includes a permuted copy of h, which no kernel writes
-  // (the gate/up GEMMs of both types gather their rows from h)
+  // fp32: the workspace is promised to hold H, Y and a permuted copy of h.  No kernel writes the copy
+  // any more: the gate/up GEMMs of both types gather their rows from h.
   if (dm.dtype == PR2_FP32) take(es * F * dm.d);
   // H [Tk, m].  The rollout routing's per-CTA histograms share its first bytes: dispatch reads
   // them before the gate/up GEMM (which waits for dispatch) writes H.

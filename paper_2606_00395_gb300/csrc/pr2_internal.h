@@ -185,12 +185,13 @@ cudaError_t launch_expert_simt(bool swiglu, const SimtArgs& g, int64_t rows, int
                                cudaStream_t st);
 
 // ---- predictive loss gradient (predictor.cu) ---------------------------------------------
-// grad_Wp = (1/T_c) G^T h_old with G = dKL/dz.  bf16: split-K tcgen05 GEMM over tokens into
-// `partial` [split, N, d] fp32, then a fixed-order reduction.  fp32: SIMT kernels.
+// grad_Wp = (1/T_c) G^T h_old with G = dKL/dz.  bf16: a tcgen05 GEMM per 128 x 128 output tile whose
+// tokens are split over the CTAs of a cluster; their fp32 partial tiles meet in `partial` and are
+// summed in rank order, in the same launch.  fp32: SIMT kernels.
 struct GradArgs {
   int N, d, Tc, Tpad;
-  int split;              // token-block split of the GEMM: CTAs per cluster (1, 2, 4 or 8)
-  float* partial;         // [split, N, d] fp32 split partials (split > 1)
+  int split;              // CTAs per cluster, any number from 1 to kLossMaxSplit
+  float* partial;         // split > 1: fp32 partial tiles [tile][rank][column / 4][row][4]
   float* grad;            // [N, d]
   const float* kl_tok;    // [Tc]
   float* loss;            // [1]

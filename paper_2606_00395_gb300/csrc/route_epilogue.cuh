@@ -1,7 +1,6 @@
-// Warp-cooperative finish of one token's routing, shared by the fp32 SIMT kernel and the
-// split-K tensor-core kernel.  The token's logits are spread over the warp: lane l holds expert
-// e = 32 j + l in zr[j] (z = p_old + b in predict mode, p in replay mode; -FLT_MAX beyond N)
-// and the router part p in pr[j].
+// Warp-cooperative finish of one token's routing in the fp32 SIMT kernel.  The token's logits are
+// spread over the warp: lane l holds expert e = 32 j + l in zr[j] (z = p_old + b in predict mode, p
+// in replay mode; -FLT_MAX beyond N) and the router part p in pr[j].
 //   predict (Eqs. pr2_predict, pr2_route): rho_hat = Softmax(z); idx = TopK(rho_hat, k) by k
 //            rounds of warp argmax (ties to the lower expert); gates = rho_hat[idx];
 //            aux = p_old row (feature-cache logits); returns whether

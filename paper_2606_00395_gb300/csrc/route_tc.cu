@@ -15,7 +15,7 @@
 // clusters are all resident at once is taken, for any N and any number of K blocks: when it had
 // to divide them (and N into sixteens) predict of 1000 tokens, d = 2048, took 25.3 us with N = 80
 // (now 9.6), 35.9 with N = 144 (13.1), 26 with N = 256 (17.5), 53.7 with N = 256 and d = 7168
-// (24.8), 29 with N = 128 and d = 2112 (11.5); loss T = 600, N = 160 28.3 (16).  With S = 2 and
+// (24.8), 29 with N = 128 and d = 2112 (11.5); loss T = 600, N = 160 27.9 (15.3).  With S = 2 and
 // N > 128 predict splits the two passes over K instead (below).  When the tiles outnumber the SMs
 // (S = 1), each CTA takes half the pipeline stages so that two run on an SM side by side, one
 // CTA's loads and finishing overlapping the other's MMAs (RouteTcArgs::compact; predict T = 32768,
@@ -57,8 +57,8 @@
 namespace pr2 {
 namespace {
 
-constexpr int kThreads = 192;                    // split = 1
-constexpr int kWarpThreads = 512;                // split > 1: rows finished by warps
+constexpr int kThreads = 192;                    // rows finished by threads
+constexpr int kWarpThreads = 512;                // rows finished by warps
 constexpr int kBK = 64;                          // bf16 elements per 128-byte swizzle row
 constexpr int kATileBytes = kTileM * kBK * 2;    // 16 KB
 constexpr int kKeep = kMaxTopK + 1;              // top-(k+1) kept for the margin
