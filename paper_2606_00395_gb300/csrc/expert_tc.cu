@@ -12,7 +12,10 @@
 // 128 B per row into shared memory for 2 x 4 MMAs of N = the rows rounded up to 16.
 //
 // What bounds it: at large experts the ~64 B per clk that an SM takes in from L2, then the power
-// limit; at ~256 rows per expert and below the weight stream from HBM.  Rows as M = 128 against N
+// limit; below ~200 rows per expert the weight stream from HBM; just above 256 rows the intake
+// again, because an expert of 270 rows is two tiles of ~136, each with its 32 KB of weights per K
+// block for half the MMAs (DeepSeek-V3-shaped launch: 4022 us at T = 7200, where 5 of 256 experts are
+// above 256 rows, 5282 at 8192, 123 of them, 7242 at 14000).  Rows as M = 128 against N
 // = 256 weight rows (the layout before) bring 48 KB per 4 MMAs of 128 x 256 x 16, 750 clk of
 // intake for 512 clk of MMA; 256 x 256 bring 64 KB per 8 of them, 1024 for 1024.  An expert of up
 // to 256 rows reads its weights from L2 once instead of 2-3 times, and N follows its row count
