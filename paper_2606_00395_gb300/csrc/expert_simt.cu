@@ -61,11 +61,8 @@ __global__ void __launch_bounds__((SimtTile<BM, BN, TM, TN, BK, kSwiglu>::kThrea
   const int r0 = (row_block % kSub) * BM;
   if (r0 >= te.rows) return;
   const int c0 = (static_cast<int>(blockIdx.x) % col_blocks) * BN;
-  // the tile's first row: of A where rows are not gathered (gate/up of a shared expert: the token;
-  // down: the H row), and of the output
-  const int64_t row0 = static_cast<uint32_t>(te.out_row0);
-  const float* A0 = kSwiglu ? (shared ? A + static_cast<int64_t>(te.a_row0) * K : A) : A + row0 * K;
-  float* out0 = g.out + row0 * n_out;
+  // row numbers are 32 unsigned bits (TileEntry); times unsigned lengths, one wide multiply each
+  const uint32_t out_row0 = static_cast<uint32_t>(te.out_row0);
   const int tid = threadIdx.x;
   const bool vec = K % 4 == 0;  // rows of 16-byte words (every base is 16-byte aligned)
 
@@ -79,8 +76,10 @@ __global__ void __launch_bounds__((SimtTile<BM, BN, TM, TN, BK, kSwiglu>::kThrea
     src[i] = A;
     if (row < BM) {
       if (r0 + row < te.rows) {
-        const int p = r0 + row;
-        src[i] = A0 + static_cast<int64_t>(kSwiglu && !shared ? g.perm[te.a_row0 + p] / g.k : p) * K + kc;
+        // gate/up: the token at this place (shared experts: the token itself); down: its H row
+        const uint32_t p = (kSwiglu ? static_cast<uint32_t>(te.a_row0) : out_row0) + (r0 + row);
+        const uint32_t at = kSwiglu && !shared ? static_cast<uint32_t>(g.perm[p] / g.k) : p;
+        src[i] = A + static_cast<uint64_t>(at) * static_cast<uint32_t>(K) + kc;
         on |= 1u << i;
       }
     } else {
@@ -175,7 +174,7 @@ __global__ void __launch_bounds__((SimtTile<BM, BN, TM, TN, BK, kSwiglu>::kThrea
   for (int i = 0; i < TM; ++i) {
     const int r = r0 + ty + kTy * i;
     if (r >= te.rows) continue;
-    float* orow = out0 + static_cast<int64_t>(r) * n_out;
+    float* orow = g.out + static_cast<uint64_t>(out_row0 + r) * static_cast<uint32_t>(n_out);
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
       const int c = c0 + tx + kTx * j;
